@@ -801,35 +801,45 @@ extern "C" int wh_kmeans_slotting(wh_layout* h, const wh_orders* orders, const i
     int rc = bind_device(h);
     if (rc != WH_OK) return rc;
     const size_t n = (size_t)o.n_sku, K = (size_t)k;
-    const size_t nb = (n + 255) / 256;
-    const size_t sz[] = {
-        align_up(8 * n * wh::KM_DIM),             // co
-        align_up(4 * n),                          // freq
-        x_out ? 0 : align_up(4 * n * wh::KM_DIM), // x
-        init ? 0 : align_up(8 * n),               // dmin
-        init ? 0 : align_up(8 * nb),              // bsum
-        align_up(4),                              // done
-        init_out ? 0 : align_up(4 * K),           // seeds
-        align_up(8 * K * wh::KM_DIM),             // sum
-        align_up(4 * K),                          // cnt
-        align_up(8 * K),                          // weight
-        align_up(4 * K),                          // off
-        align_up(4 * K),                          // cur
-        align_up(4 * (K + 1)),                    // off_by_rank
-        align_up(8 * n),                          // mkey
-    };
-    size_t total = 0;
-    for (size_t v : sz) total += v;
-    rc = reserve_scratch(h, total);
-    if (rc != WH_OK) return rc;
-    char* q = static_cast<char*>(h->scratch);
-    auto take = [&](size_t bytes) -> void* {
-        void* r = bytes ? q : nullptr;
-        q += bytes;
-        return r;
-    };
+    const size_t nb = (n + 255) / 256, tiles = (n + 1023) / 1024;
+    // more ordered SKUs (at most the lines, at most all) than a cluster holds:
+    // a launch per seed, with its distances in global memory
+    const bool rounds = !init && std::min(o.n_sku, o.n_lines) > wh::kmeans_pp_rows();
     wh::KmArgs A;
     std::memset(&A, 0, sizeof(A));
+    char* q = nullptr;
+    auto take = [&](size_t bytes) -> void* {
+        void* r = bytes ? q : nullptr;
+        q += align_up(bytes);
+        return r;
+    };
+    auto lay_out = [&](char* base) {
+        q = base;
+        A.co = static_cast<long long*>(take(8 * n * wh::KM_DIM));
+        A.freq = static_cast<int32_t*>(take(4 * n));
+        A.sum = static_cast<long long*>(take(8 * K * wh::KM_DIM));
+        A.cnt = static_cast<int32_t*>(take(4 * K));
+        A.weight = static_cast<long long*>(take(8 * K));
+        A.done = static_cast<unsigned int*>(take(4));
+        A.max_freq = static_cast<unsigned int*>(take(4));
+        A.zeroed = base;
+        A.zeroed_bytes = (size_t)(q - base);
+        A.x = x_out ? x_out : static_cast<int32_t*>(take(4 * n * wh::KM_DIM));
+        A.dmin = static_cast<long long*>(take(rounds ? 8 * n : 0));
+        A.bsum = static_cast<long long*>(take(rounds ? 8 * nb : 0));
+        A.seeds = init_out ? init_out : static_cast<int32_t*>(take(4 * K));
+        A.bcount = static_cast<int32_t*>(take(4 * nb));
+        A.active = static_cast<int32_t*>(take(4 * n));
+        A.n_active = static_cast<int32_t*>(take(4));
+        A.rank = static_cast<int32_t*>(take(4 * K));
+        A.order_a = static_cast<int32_t*>(take(4 * n));
+        A.order_b = static_cast<int32_t*>(take(4 * n));
+        A.rs_count = static_cast<int32_t*>(take(4 * 256 * tiles));
+        return (size_t)(q - base);
+    };
+    rc = reserve_scratch(h, lay_out(reinterpret_cast<char*>(kAlign)));   // (measured from any aligned base)
+    if (rc != WH_OK) return rc;
+    lay_out(static_cast<char*>(h->scratch));
     A.g = h->g;
     A.n_orders = o.n_orders;
     A.n_lines = o.n_lines;
@@ -842,21 +852,7 @@ extern "C" int wh_kmeans_slotting(wh_layout* h, const wh_orders* orders, const i
     A.iters = iters;
     A.init = init;
     A.u = u;
-    A.co = static_cast<long long*>(take(sz[0]));
-    A.freq = static_cast<int32_t*>(take(sz[1]));
-    A.x = x_out ? x_out : static_cast<int32_t*>(take(sz[2]));
-    A.dmin = static_cast<long long*>(take(sz[3]));
-    A.bsum = static_cast<long long*>(take(sz[4]));
-    A.done = static_cast<unsigned int*>(take(sz[5]));
-    A.seeds = init_out ? init_out : static_cast<int32_t*>(take(sz[6]));
     A.cent = centroids;
-    A.sum = static_cast<long long*>(take(sz[7]));
-    A.cnt = static_cast<int32_t*>(take(sz[8]));
-    A.weight = static_cast<long long*>(take(sz[9]));
-    A.off = static_cast<int32_t*>(take(sz[10]));
-    A.cur = static_cast<int32_t*>(take(sz[11]));
-    A.off_by_rank = static_cast<int32_t*>(take(sz[12]));
-    A.mkey = static_cast<unsigned long long*>(take(sz[13]));
     A.assign = assign;
     A.slot_map = slot_map;
     A.status = h->meta;

@@ -201,26 +201,34 @@ struct KmArgs {
     int32_t fw, k, iters;
     const int32_t* init;         // [k] or null: K-means++ from u
     const uint64_t* u;           // [k]
-    long long* co;               // [n_sku][32] scratch
+    // scratch that starts at zero, in one block: co, freq, sum, cnt, weight,
+    // the finished-block ticket and the largest pick count
+    void* zeroed;
+    size_t zeroed_bytes;
+    long long* co;               // [n_sku][32]
     int32_t* freq;               // [n_sku]
-    int32_t* x;                  // [n_sku][32]
-    long long* dmin;             // [n_sku]
-    long long* bsum;             // [blocks]
-    unsigned int* done;
-    int32_t* seeds;              // [k]
-    int32_t* cent;               // [k][32]
     long long* sum;              // [k][32]
     int32_t* cnt;                // [k]
     long long* weight;           // [k]
-    int32_t* off;                // [k]
-    int32_t* cur;                // [k]
-    int32_t* off_by_rank;        // [k + 1]
-    unsigned long long* mkey;    // [n_sku]
+    unsigned int* done;
+    unsigned int* max_freq;
+    int32_t* x;                  // [n_sku][32]
+    long long* dmin;             // [n_sku]; null: one cluster seeds
+    long long* bsum;             // [blocks], with dmin
+    int32_t* seeds;              // [k]
+    int32_t* cent;               // [k][32]
+    int32_t* bcount;             // [blocks] ordered SKUs per block of 256
+    int32_t* active;             // [n_sku] the ordered SKUs, ascending
+    int32_t* n_active;
+    int32_t* rank;               // [k] cluster ranks by weight
+    int32_t* order_a;            // [n_sku] the zones' sort, ping-pong
+    int32_t* order_b;
+    int32_t* rs_count;           // [256][tiles of 1,024 SKUs]
     int32_t* assign;             // [n_sku]
     int32_t* slot_map;           // [n_sku]
     uint32_t* status;
 };
-size_t kmeans_assign_smem(int k);
+int kmeans_pp_rows();   // ordered SKUs up to which one cluster seeds
 cudaError_t launch_kmeans(const KmArgs& A, cudaStream_t s);
 
 // explicit optimal routes of listed tours (k_route.cu)
