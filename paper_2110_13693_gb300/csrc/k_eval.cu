@@ -149,27 +149,6 @@ __device__ __forceinline__ void warp_chunk_range(const EvalArgs& a, int& c_begin
     c_end = (int)((gw + 1) * n_chunks / warps);
 }
 
-// Plan of tour t0 (the largest p with plan_tour_off[p] <= t0), found by the
-// whole warp: each round probes 32 evenly spaced offsets of the remaining
-// range at once and keeps the piece between the last probe at or below t0
-// and the next, so the range shrinks 32-fold per round (3 dependent loads
-// for 4,096 plans instead of 12).  Every lane returns the same plan.
-__device__ __forceinline__ int warp_find_plan(const EvalArgs& a, int t0, int lane) {
-    int lo = 0, hi = a.n_plans - 1;
-    while (lo < hi) {
-        const int span = hi - lo;                         // candidates lo+1 .. hi
-        const int idx = lo + (int)(((int64_t)span * (lane + 1) + 31) / 32);   // in [lo+1, hi], non-decreasing
-        const bool le = a.plan_tour_off[idx] <= t0;
-        const unsigned below = __ballot_sync(0xffffffffu, le);   // a prefix of the lanes
-        const int k = __popc(below);
-        const int lo_new = k ? __shfl_sync(0xffffffffu, idx, k - 1) : lo;
-        const int hi_new = k < 32 ? __shfl_sync(0xffffffffu, idx, k < 32 ? k : 31) - 1 : hi;
-        lo = lo_new;
-        hi = hi_new;
-    }
-    return lo;
-}
-
 // One warp scores the 32-tour chunks [c_begin, c_end) of instance `a`, one
 // tour per lane, and adds its plans' sums with one atomic per plan segment.
 template <bool KEY16, bool SHARED_MAP, bool SMEM_TABLES, bool ID16 = false>
