@@ -857,11 +857,19 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_eval_long(LongArgs L) {
                 const int q = qb + lane;
                 int lb = 0, le = 0;
                 if (q < q1) {
-                    // in range: checked by the short kernel
+                    // checked here: the short kernel hands the tour over at
+                    // the order that takes it past its lines, before it has
+                    // seen the ones behind
                     const int o = qb == q0 ? o_first : id_of(inst, q);
-                    lb = a.order_off[o];
-                    le = a.order_off[o + 1];
-                    if (lb < 0 || le < lb || le > a.n_lines) {
+                    const bool in = (unsigned)o < (unsigned)a.n_orders;
+                    if (in) {
+                        lb = a.order_off[o];
+                        le = a.order_off[o + 1];
+                    }
+                    if (!in) {
+                        flag(a.status, WH_STATUS_BAD_ORDER);
+                        bad = true;
+                    } else if (lb < 0 || le < lb || le > a.n_lines) {
                         flag(a.status, WH_STATUS_BAD_OFFSET);
                         bad = true;
                         lb = le = 0;
