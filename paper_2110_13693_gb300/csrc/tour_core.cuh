@@ -187,20 +187,25 @@ __device__ __forceinline__ int sshape_cost(const Geo& g, int m, int last_a, int 
 }
 
 // ------------------------------------------------------ 32-bit key network
-template <int N>
-__device__ __forceinline__ void bitonic_sort(uint32_t (&x)[N]) {
+// Ascending sort of the first N registers by Batcher's merge exchange (Knuth,
+// TAOCP vol. 3, Algorithm 5.2.2M), fully unrolled: for 64 keys 543
+// comparators where the bitonic network takes 672.  N need not be a power of
+// two; registers from N on are left alone.
+template <int N, int M>
+__device__ __forceinline__ void merge_exchange(uint32_t (&x)[M]) {
+    static_assert(N <= M && N <= 128, "keys in registers");
+    constexpr int T = N > 64 ? 64 : N > 32 ? 32 : N > 16 ? 16 : N > 8 ? 8 : N > 4 ? 4 : N > 2 ? 2 : 1;
 #pragma unroll
-    for (int k = 2; k <= N; k <<= 1) {
+    for (int p = T; p > 0; p >>= 1) {
 #pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int q = T; q >= p; q >>= 1) {
+            const int r = q == T ? 0 : p, d = q == T ? p : 2 * q - p;
 #pragma unroll
             for (int i = 0; i < N; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const uint32_t a = x[i], b = x[l];
-                    const uint32_t lo = min(a, b), hi = max(a, b);
-                    if ((i & k) == 0) { x[i] = lo; x[l] = hi; }
-                    else { x[i] = hi; x[l] = lo; }
+                if (i + d < N && (i & p) == r) {
+                    const uint32_t a = x[i], b = x[i + d];
+                    x[i] = min(a, b);
+                    x[i + d] = max(a, b);
                 }
             }
         }
@@ -209,47 +214,45 @@ __device__ __forceinline__ void bitonic_sort(uint32_t (&x)[N]) {
 
 // ------------------------------------------------------ 16-bit key network
 // 2R positions in R registers: position p lives in register p % R, in the low
-// half when p < R and the high half otherwise.  All-ascending bitonic sorter:
-// each merge of block size k starts by comparing p with p ^ (k-1) (the
-// mirrored partner), then half-cleans with p ^ j for j = k/4 .. 1.  For
-// k <= R both halves run the same register pairs, so one 16x2 min/max pair
-// serves two comparators; the final mirror step pairs halves across
-// registers and needs a half swap.
+// half when p < R and the high half otherwise.  Both halves are sorted by the
+// same register pairs (merge_exchange's comparators, one 16x2 min/max pair
+// for two of them: 191 pairs for R = 32, where a bitonic sort of the halves
+// takes 240), then merged: p against its mirror p ^ (2R - 1), a half swap
+// across registers, and half-cleaners p ^ j for j = R/2 .. 1.
 template <int R>
 __device__ __forceinline__ void sort16x2(uint32_t (&x)[R]) {
-    constexpr int N = 2 * R;
 #pragma unroll
-    for (int k = 2; k <= N; k <<= 1) {
-        if (k == N) {
+    for (int p = R / 2; p > 0; p >>= 1) {
 #pragma unroll
-            for (int r = 0; r < R / 2; ++r) {
-                const uint32_t A = x[r], B = x[R - 1 - r];
-                const uint32_t Bs = __byte_perm(B, 0, 0x1032);
-                const uint32_t mn = __vminu2(A, Bs), mx = __vmaxu2(A, Bs);
-                x[r] = __byte_perm(mn, mx, 0x7610);
-                x[R - 1 - r] = __byte_perm(mn, mx, 0x5432);
-            }
-        } else {
+        for (int q = R / 2; q >= p; q >>= 1) {
+            const int r = q == R / 2 ? 0 : p, d = q == R / 2 ? p : 2 * q - p;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int l = r ^ (k - 1);
-                if (l > r) {
-                    const uint32_t a = x[r], b = x[l];
-                    x[r] = __vminu2(a, b);
-                    x[l] = __vmaxu2(a, b);
+            for (int i = 0; i < R; ++i) {
+                if (i + d < R && (i & p) == r) {
+                    const uint32_t a = x[i], b = x[i + d];
+                    x[i] = __vminu2(a, b);
+                    x[i + d] = __vmaxu2(a, b);
                 }
             }
         }
+    }
 #pragma unroll
-        for (int j = k >> 2; j > 0; j >>= 1) {
+    for (int r = 0; r < R / 2; ++r) {
+        const uint32_t A = x[r], B = x[R - 1 - r];
+        const uint32_t Bs = __byte_perm(B, 0, 0x1032);
+        const uint32_t mn = __vminu2(A, Bs), mx = __vmaxu2(A, Bs);
+        x[r] = __byte_perm(mn, mx, 0x7610);
+        x[R - 1 - r] = __byte_perm(mn, mx, 0x5432);
+    }
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int l = r ^ j;
-                if (l > r) {
-                    const uint32_t a = x[r], b = x[l];
-                    x[r] = __vminu2(a, b);
-                    x[l] = __vmaxu2(a, b);
-                }
+    for (int j = R / 2; j > 0; j >>= 1) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int l = r ^ j;
+            if (l > r) {
+                const uint32_t a = x[r], b = x[l];
+                x[r] = __vminu2(a, b);
+                x[l] = __vmaxu2(a, b);
             }
         }
     }
@@ -458,7 +461,7 @@ __device__ __forceinline__ void tour32(const EvalArgs& a, uint2* col, int T, int
         for (int p = 0; p < N; ++p) b |= x[p] == KEY_BAD;
         *kbad = b;
     }
-    bitonic_sort<N>(x);
+    merge_exchange<N>(x);
     int last_a, last_hi;
     scan32<N>(x, col_sa, slot_b, a.max_rec, need_rr, m, last_a, last_hi);
     cs = sshape_cost(a.g, m, last_a, last_hi);
