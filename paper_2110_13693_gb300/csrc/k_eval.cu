@@ -478,6 +478,18 @@ __device__ __forceinline__ void prep_instance(const EvalArgs& a, uint32_t mask, 
     }
     if (a.order_agg)
         for (int o = i0; o < a.n_orders; o += stride) a.order_agg[o] = order_aggregate(a, o);
+    if (a.line_ord) {
+        for (int o = i0; o < a.n_orders; o += stride) {
+            // malformed offsets and orders of 255 lines or more: k_eval_plan
+            // does not read the table then
+            const int lb = a.order_off[o], le = a.order_off[o + 1];
+            if (lb >= 0 && le <= a.n_lines)
+                for (int l = lb; l < le; ++l) a.line_ord[l] = ((uint32_t)o << 8) | ((uint32_t)(l - lb) & 0xFFu);
+        }
+        const int l0 = a.n_orders > 0 ? a.order_off[0] : 0, l1 = a.n_orders > 0 ? a.order_off[a.n_orders] : 0;
+        for (int l = i0; l < a.n_lines; l += stride)
+            if (l < l0 || l >= l1) a.line_ord[l] = 0xFFFFFFFFu;
+    }
     const bool zs = a.plan_s && (mask & WH_ROUTE_SSHAPE);
     const bool zr = a.plan_rr && (mask & WH_ROUTE_OPTIMAL);
     for (int p = i0; p < a.n_plans; p += stride) {
@@ -1104,7 +1116,7 @@ static cudaError_t launch_sshape(const EvalArgs& a, const Tuning& t, int num_sms
 cudaError_t launch_prep(const EvalArgs& a, cudaStream_t s) {
     int work = a.n_plans;
     if (a.line_key && a.n_lines > work) work = a.n_lines;
-    if (a.order_agg && a.n_orders > work) work = a.n_orders;
+    if ((a.order_agg || a.line_ord) && a.n_orders > work) work = a.n_orders;
     int grid = (work + 255) / 256;
     if (grid > 4096) grid = 4096;
     if (grid < 1) grid = 1;

@@ -1,0 +1,396 @@
+// Plan evaluation with one CTA per plan, for plans that each have their own
+// slotting and for layouts whose keys need 32 bits.
+//
+// k_eval_short walks each tour's orders straight into the plan's slotting in
+// global memory: chains of dependent loads with few warps to hide them, 32
+// keys or more a thread in registers, and a separate pass of one warp a tour
+// for tours of more than 64 lines or 32 aisles.  Here a CTA takes a plan
+// through short phases of few registers each:
+//   count      a thread per tour: its orders checked and counted, a row of
+//              shared memory for its keys and every order's place in it;
+//   translate  a thread per order-book line, in line order: SKU (coalesced),
+//              its location under the plan's slotting (eight independent
+//              gathers in flight) and the key written to the order's place;
+//   sort       2, 4 or 8 lanes a tour with 16 keys each: a merge-exchange
+//              network in the lane, bitonic merges across lanes by shuffles;
+//   cost       a thread per tour, ordered by line count: one pass over the
+//              sorted row, a DP step where an aisle ends (no record slots,
+//              so no limit on a tour's aisles).
+#include "tour_core.cuh"
+
+namespace wh {
+namespace {
+
+constexpr int PL_THREADS = 256;
+constexpr int PL_CTAS = 3;       // per SM
+constexpr int PL_MAXN = 128;     // lines of a tour (8 lanes of 16); longer ones go to the long-tour pass
+constexpr int PL_LIST = 1024;    // tours of a plan taken per round
+constexpr int PL_U = PL_LIST / PL_THREADS;
+
+// Markers of unusable lines (a key's aisle is at most 65,533, so both compare
+// above every key); KEY_BAD: location out of range.
+constexpr uint32_t KEY_BAD_SKU = 0xFFFFFFFDu;
+
+// Line count of tour t, its orders checked: -1 for invalid offsets or ids
+// (flagged), PL_MAXN + 1 for a tour that the long-tour pass takes.  Four
+// order ids in flight.
+__device__ __forceinline__ int count_lines(const EvalArgs& a, const uint8_t* s_cnt, int t, int& q0, int& q1) {
+    q0 = __ldg(a.tour_off + t);
+    q1 = __ldg(a.tour_off + t + 1);
+    if (q0 < 0 || q1 < q0 || (int64_t)q1 > a.n_seq) {
+        flag(a.status, WH_STATUS_BAD_OFFSET);
+        return -1;
+    }
+    int n = 0;
+    bool bad = false;
+    for (int q = q0; q < q1; q += 4) {
+        int o[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) o[u] = q + u < q1 ? __ldg(a.order_seq + q + u) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if ((unsigned)o[u] < (unsigned)a.n_orders) n += s_cnt[o[u]];
+            else bad |= q + u < q1;
+        }
+        n = min(n, PL_MAXN + 1);
+    }
+    if (bad) {
+        flag(a.status, WH_STATUS_BAD_ORDER);
+        return -1;
+    }
+    return n;
+}
+
+// Sort the rows of tours list[i0 + lane / G] (those below i1), G lanes a tour
+// with 16 keys each.
+template <int G>
+__device__ __forceinline__ void sort_rows(uint32_t* rows, const uint16_t* s_list, const uint16_t* s_base,
+                                          const uint8_t* s_n, int i0, int i1, int lane) {
+    const int sub = lane & (G - 1), i = i0 + lane / G;
+    int n = 0;
+    uint32_t* row = rows;
+    if (i < i1) {
+        const int k = s_list[i];
+        n = s_n[k];
+        row = rows + s_base[k];
+    }
+    uint32_t x[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) x[j] = j * G + sub < n ? row[j * G + sub] : KEY_NONE;
+    merge_exchange<16>(x);
+#pragma unroll
+    for (int s = 1; s < G; s <<= 1) {
+        // blocks of s lanes merged in pairs: every key against its mirror
+        const bool low = (lane & s) == 0;
+        uint32_t y[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) y[j] = __shfl_xor_sync(0xffffffffu, x[15 - j], 2 * s - 1);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) x[j] = low ? min(x[j], y[j]) : max(x[j], y[j]);
+#pragma unroll
+        for (int d = s >> 1; d > 0; d >>= 1) {
+            const bool l2 = (lane & d) == 0;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const uint32_t o = __shfl_xor_sync(0xffffffffu, x[j], d);
+                x[j] = l2 ? min(x[j], o) : max(x[j], o);
+            }
+        }
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                if ((j ^ d) > j) {
+                    const uint32_t p = x[j], r = x[j ^ d];
+                    x[j] = min(p, r);
+                    x[j ^ d] = max(p, r);
+                }
+            }
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+        if (sub * 16 + j < n) row[sub * 16 + j] = x[j];
+}
+
+// sum over the warp's lanes of values 0 <= v < 2^31
+__device__ __forceinline__ long long warp_sum31(int v) {
+    const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)v >> 16);
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xFFFFu);
+    return ((long long)hi << 16) + lo;
+}
+
+template <bool SHARED_MAP>
+__global__ void __launch_bounds__(PL_THREADS, PL_CTAS) k_eval_plan(EvalArgs a) {
+    extern __shared__ __align__(16) uint32_t rows[];   // keys, then per order: place, line count, seen bit
+    __shared__ int s_bin[PL_MAXN + 1];        // tours of every line count, then their first place in the list
+    __shared__ uint16_t s_list[PL_LIST];      // the round's tours by falling line count
+    __shared__ uint16_t s_base[PL_LIST];      // their rows, by tour
+    __shared__ uint8_t s_n[PL_LIST];          // their line counts, by tour
+    __shared__ int s_total, s_unit, s_rows, s_dup;
+    const int tid = threadIdx.x, lane = tid & 31;
+    constexpr int T = PL_THREADS;
+    uint32_t* s_dst32 = rows + a.n_lines;     // first place of an order's lines, 16 bits each (0xFFFF: none)
+    uint16_t* s_dst = reinterpret_cast<uint16_t*>(s_dst32);
+    const int n_dst = (a.n_orders + 1) >> 1, n_seen = (a.n_orders + 31) >> 5;
+    uint32_t* s_seen = s_dst32 + n_dst;
+    uint8_t* s_cnt = reinterpret_cast<uint8_t*>(s_seen + n_seen);
+    const bool need_rr = (a.mask & WH_ROUTE_OPTIMAL) != 0;
+    const bool want_s = (a.mask & WH_ROUTE_SSHAPE) != 0;
+
+    // line counts; an order book with malformed offsets or an order of 255
+    // lines or more has no line -> order table to go by
+    bool odd = false;
+    for (int o = tid; o < a.n_orders; o += T) {
+        const int lb = a.order_off[o], le = a.order_off[o + 1];
+        const bool ok = lb >= 0 && le >= lb && le <= a.n_lines && le - lb < 255;
+        s_cnt[o] = ok ? (uint8_t)(le - lb) : 0;
+        odd |= !ok;
+    }
+    odd = __syncthreads_or(odd);
+
+    for (int plan = blockIdx.x; plan < a.n_plans; plan += gridDim.x) {
+        const int32_t* map = SHARED_MAP ? nullptr : a.slot_map + (int64_t)plan * a.slot_stride;
+        // k_prep has flagged malformed plan offsets
+        const int t0 = max(a.plan_tour_off[plan], 0), t1 = min(a.plan_tour_off[plan + 1], a.n_tours);
+        for (int tb = t0; tb < t1; tb += PL_LIST) {
+            const int nt = min(PL_LIST, t1 - tb);
+            for (int i = tid; i <= PL_MAXN; i += T) s_bin[i] = 0;
+            for (int i = tid; i < n_dst; i += T) s_dst32[i] = 0xFFFFFFFFu;
+            for (int i = tid; i < n_seen; i += T) s_seen[i] = 0u;
+            if (tid == 0) s_unit = s_rows = s_dup = 0;
+            __syncthreads();
+            // ---- count
+            int at[PL_U];   // place in the tour's bin, -1: not scored here
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u) {
+                const int i = tid + u * T;
+                at[u] = -1;
+                if (i >= nt) continue;
+                int q0, q1;
+                const int n = count_lines(a, s_cnt, tb + i, q0, q1);
+                if (n < 0) {
+                    if (a.tour_s) a.tour_s[tb + i] = -1;
+                    if (a.tour_rr) a.tour_rr[tb + i] = -1;
+                    continue;
+                }
+                s_n[i] = (uint8_t)min(n, 255);
+                at[u] = 0;
+                if (odd || n > PL_MAXN) continue;
+                int pos = atomicAdd(&s_rows, n);
+                if (pos + n > a.n_lines) {   // more lines than the book has: an order is taken twice
+                    s_dup = 1;
+                    continue;
+                }
+                s_base[i] = (uint16_t)pos;
+                at[u] = atomicAdd(&s_bin[n], 1);
+                for (int q = q0; q < q1; q += 4) {
+                    int o[4];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) o[v] = q + v < q1 ? __ldg(a.order_seq + q + v) : -1;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        if (o[v] < 0) continue;
+                        const uint32_t bit = 1u << (o[v] & 31);
+                        if (atomicOr(&s_seen[o[v] >> 5], bit) & bit) s_dup = 1;
+                        s_dst[o[v]] = (uint16_t)pos;
+                        pos += s_cnt[o[v]];
+                    }
+                }
+            }
+            __syncthreads();
+            const bool all_long = odd || s_dup;
+            // tours that the long-tour pass takes: too many lines, or (all of
+            // them) an order book or a plan whose lines have no single place
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u) {
+                const int i = tid + u * T;
+                if (at[u] < 0 || !(all_long || s_n[i] > PL_MAXN)) continue;
+                at[u] = -1;
+                const int slot = atomicAdd(a.long_count, 1);
+                if (slot < a.long_cap) {
+                    a.long_list[3 * slot] = 0;
+                    a.long_list[3 * slot + 1] = tb + i;
+                    a.long_list[3 * slot + 2] = plan;
+                } else {
+                    flag(a.status, WH_STATUS_LONG_OVERFLOW);
+                    if (a.tour_s) a.tour_s[tb + i] = -1;
+                    if (a.tour_rr) a.tour_rr[tb + i] = -1;
+                }
+            }
+            if (all_long) {
+                __syncthreads();   // s_dup is reset next
+                continue;
+            }
+            // the bins' first places in the list: most lines first
+            if (tid < 32) {
+                constexpr int B = (PL_MAXN + 32) / 32;
+                int v[B], sum = 0;
+#pragma unroll
+                for (int u = 0; u < B; ++u) {
+                    const int b = PL_MAXN - (B * lane + u);
+                    v[u] = b >= 0 ? s_bin[b] : 0;
+                    sum += v[u];
+                }
+                const int incl = warp_inclusive_scan(sum);
+                int pos = incl - sum;
+#pragma unroll
+                for (int u = 0; u < B; ++u) {
+                    const int b = PL_MAXN - (B * lane + u);
+                    if (b >= 0) s_bin[b] = pos;
+                    pos += v[u];
+                }
+                if (lane == 31) s_total = incl;
+            }
+            // ---- translate
+            for (int l0 = tid; l0 < a.n_lines; l0 += 8 * T) {
+                uint32_t sk[8], at_o[8];
+                int loc[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int l = l0 + u * T;
+                    sk[u] = l < a.n_lines ? (SHARED_MAP ? a.line_key[l] : (uint32_t)__ldg(a.line_sku + l)) : 0u;
+                    at_o[u] = l < a.n_lines ? a.line_ord[l] : 0xFFFFFFFFu;
+                }
+                if constexpr (!SHARED_MAP) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) loc[u] = sk[u] < (uint32_t)a.n_sku ? __ldg(map + sk[u]) : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (at_o[u] == 0xFFFFFFFFu) continue;   // past the end, or in no order
+                    const uint32_t d = s_dst[at_o[u] >> 8];
+                    if (d == 0xFFFFu) continue;             // in none of the round's tours
+                    uint32_t k = sk[u];
+                    if constexpr (!SHARED_MAP) {
+                        k = loc_key(a.g, loc[u]);
+                        if ((uint32_t)loc[u] >= (uint32_t)a.g.n_loc) k = KEY_BAD;
+                        if (sk[u] >= (uint32_t)a.n_sku) k = KEY_BAD_SKU;
+                    }
+                    rows[d + (at_o[u] & 0xFFu)] = k;
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < PL_U; ++u)
+                if (at[u] >= 0) s_list[s_bin[s_n[tid + u * T]] + at[u]] = (uint16_t)(tid + u * T);
+            __syncthreads();
+            // ---- sort: units of a warp's tours, the longest first
+            const int total = s_total, c8 = s_bin[64], c4 = s_bin[32];   // tours over 64 and over 32 lines
+            const int u8n = (c8 + 3) >> 2, u4n = u8n + ((c4 - c8 + 7) >> 3), un = u4n + ((total - c4 + 15) >> 4);
+            for (;;) {
+                int u = lane == 0 ? atomicAdd(&s_unit, 1) : 0;
+                u = __shfl_sync(0xffffffffu, u, 0);
+                if (u >= un) break;
+                if (u < u8n) sort_rows<8>(rows, s_list, s_base, s_n, 4 * u, c8, lane);
+                else if (u < u4n) sort_rows<4>(rows, s_list, s_base, s_n, c8 + 8 * (u - u8n), c4, lane);
+                else sort_rows<2>(rows, s_list, s_base, s_n, c4 + 16 * (u - u4n), total, lane);
+            }
+            __syncthreads();
+            // ---- cost
+            const DPConst c = dp_const(a.g);
+            for (int i0 = tid & ~31; i0 < total; i0 += T) {
+                const bool on = i0 + lane < total;
+                const int k = on ? s_list[i0 + lane] : 0, t = tb + k, n = on ? s_n[k] : 0;
+                const uint32_t* row = rows + (on ? s_base[k] : 0);
+                DP5 v;
+                dp_init(v);
+                int pa = 0, m = 0;
+                uint32_t key = n > 0 ? row[0] : 0u, lo = key, gi = 0, last = 0;
+                for (int p = 0; p < n; p += 4) {
+                    uint32_t nx[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) nx[j] = p + j + 1 < n ? row[p + j + 1] : KEY_NONE;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (nx[j] > (key | 0xFFFFu)) {
+                            const int ai = (int)(key >> 16);
+                            if (need_rr)
+                                dp_aisle_rel(v, c, ai - pa, (int)(lo & 0xFFFFu), (int)(key & 0xFFFFu), (int)gi);
+                            pa = ai;
+                            ++m;
+                            last = key;
+                            lo = nx[j];
+                            gi = 0;
+                        } else {
+                            gi = max(gi, nx[j] - key);
+                        }
+                        key = nx[j];
+                    }
+                }
+                // markers sort last and never end an aisle
+                const bool kbad = n > 0 && row[n - 1] >= KEY_BAD_SKU;
+                const int cs = sshape_cost(a.g, m, (int)(last >> 16), (int)(last & 0xFFFFu));
+                const int cr = need_rr ? dp_final(v) + c.p2 * pa : 0;
+                if (kbad) {
+                    if constexpr (!SHARED_MAP)   // under a shared slotting k_prep has flagged the line
+                        for (int p = n - 1; p >= 0 && row[p] >= KEY_BAD_SKU; --p)
+                            flag(a.status, row[p] == KEY_BAD ? WH_STATUS_BAD_LOC : WH_STATUS_BAD_SKU);
+                    if (a.tour_s) a.tour_s[t] = -1;
+                    if (a.tour_rr) a.tour_rr[t] = -1;
+                } else if (on) {
+                    if (a.tour_s && want_s) a.tour_s[t] = cs;
+                    if (a.tour_rr && need_rr) a.tour_rr[t] = cr;
+                }
+                const bool ok = on && !kbad;
+                const long long ss = warp_sum31(ok ? cs : 0), sr = warp_sum31(ok ? cr : 0);
+                if (lane == 0) {
+                    if (a.plan_s && want_s && ss)
+                        atomicAdd(reinterpret_cast<unsigned long long*>(&a.plan_s[plan]), (unsigned long long)ss);
+                    if (a.plan_rr && need_rr && sr)
+                        atomicAdd(reinterpret_cast<unsigned long long*>(&a.plan_rr[plan]), (unsigned long long)sr);
+                }
+            }
+            __syncthreads();   // the rows are about to be rewritten
+        }
+    }
+}
+
+size_t plan_smem_bytes(const EvalArgs& a) {
+    return sizeof(uint32_t) * ((size_t)a.n_lines + ((size_t)a.n_orders + 1) / 2 + ((size_t)a.n_orders + 31) / 32) +
+           (((size_t)a.n_orders + 15) & ~(size_t)15);
+}
+
+}  // namespace
+
+// Measured against k_eval_short + k_eval_long (us a call, GB300; orders x
+// tours a plan x lines a tour):
+//   own slottings    4,000 x 167 x 59, 500 aisles: 16 plans 58 -> 35,
+//                    500 plans 167 -> 68, 2,000 plans 516 -> 202
+//                    4,000 x 200 x 49, 40 aisles: 16 plans 58 -> 32,
+//                    2,000 plans 238 -> 156
+//                    300 x 38 x 20: 500 plans 33 -> 27, 2,000 plans 40 -> 50
+//                    400 x 17 x 59: 500 plans 54 -> 38, 2,000 plans 82 -> 77
+//   shared, 32-bit   4,000 x 167 x 59: 16 plans 46 -> 33, 2,000 plans 334 -> 153
+//                    400 x 17 x 59: 152 plans 37 -> 25, 2,000 plans 50 -> 72
+//                    3,000 x 375 x 20: 64 plans 25 -> 29, 152 plans 29 -> 29,
+//                    2,000 plans 206 -> 113
+// So: many plans of few tours (a CTA's threads idle, and one tour per thread
+// fills the chip anyway) and few plans of short tours under a shared slotting
+// (k_eval_short has no latency of gathers or of a long-tour pass there) stay.
+// Three CTAs an SM take order books of up to 67 KB; a shared slotting with
+// 16-bit keys is k_eval_short's best case (half the sort, one gather).
+bool eval_plan_applies(const EvalArgs& a, int num_sms) {
+    if (sshape_kernel_applies(a) || a.n_tours == 0 || a.n_lines > 0xFFFE || plan_smem_bytes(a) > 67 * 1024) return false;
+    if (a.n_plans > 4 * num_sms && a.n_tours / a.n_plans < 64) return false;
+    if (a.slot_stride != 0) return true;
+    if (key16_ok(a.g)) return false;
+    return a.n_plans >= num_sms || (double)a.n_lines * (double)a.n_seq > 32.0 * (double)a.n_orders * (double)a.n_tours;
+}
+
+cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s) {
+    const size_t smem = plan_smem_bytes(a);
+    auto kern = a.slot_stride == 0 ? k_eval_plan<true> : k_eval_plan<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PL_THREADS, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    const int grid = a.n_plans < per_sm * num_sms ? a.n_plans : per_sm * num_sms;
+    kern<<<grid, PL_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace wh

@@ -317,15 +317,18 @@ extern "C" int wh_eval_plans(wh_layout* h, const wh_orders* orders, const wh_pla
     const bool agg = shared_map && routing_mask == WH_ROUTE_SSHAPE && h->g.A <= 64 && o.n_orders > 0;
     const size_t key_bytes = shared_map && !agg ? align_up(sizeof(uint32_t) * (size_t)o.n_lines) : 0;
     const size_t agg_bytes = agg ? align_up(sizeof(uint4) * (size_t)o.n_orders) : 0;
+    const bool per_plan = wh::eval_plan_applies(a, h->num_sms);
+    const size_t ord_bytes = per_plan ? align_up(sizeof(uint32_t) * (size_t)o.n_lines) : 0;
     const size_t list_bytes = align_up(sizeof(int32_t) * 3 * ((size_t)p.n_tours + 1));
     const size_t rec_bytes = align_up(wh::long_rec_bytes(h->num_sms));
-    rc = reserve_scratch(h, key_bytes + agg_bytes + list_bytes + rec_bytes);
+    rc = reserve_scratch(h, key_bytes + agg_bytes + list_bytes + rec_bytes + ord_bytes);
     if (rc != WH_OK) return rc;
     char* base = static_cast<char*>(h->scratch);
     a.line_key = shared_map && !agg && o.n_lines > 0 ? reinterpret_cast<uint32_t*>(base) : nullptr;
     a.order_agg = agg ? reinterpret_cast<uint4*>(base + key_bytes) : nullptr;
     a.long_list = reinterpret_cast<int32_t*>(base + key_bytes + agg_bytes);
     uint2* long_rec = rec_bytes ? reinterpret_cast<uint2*>(base + key_bytes + agg_bytes + list_bytes) : nullptr;
+    a.line_ord = ord_bytes ? reinterpret_cast<uint32_t*>(base + key_bytes + agg_bytes + list_bytes + rec_bytes) : nullptr;
 
     {
         LaunchTimer lt(h->timing, K_PREP, s);
@@ -333,7 +336,10 @@ extern "C" int wh_eval_plans(wh_layout* h, const wh_orders* orders, const wh_pla
     }
     {
         LaunchTimer lt(h->timing, wh::sshape_kernel_applies(a) ? K_EVAL_SSHAPE : K_EVAL_SHORT, s);
-        if (!lt.ok() || wh::launch_eval_short(a, t, h->num_sms, s, nullptr) != cudaSuccess) return WH_ECUDA;
+        if (!lt.ok()) return WH_ECUDA;
+        const cudaError_t e = per_plan ? wh::launch_eval_plan(a, h->num_sms, s)
+                                       : wh::launch_eval_short(a, t, h->num_sms, s, nullptr);
+        if (e != cudaSuccess) return WH_ECUDA;
     }
     // the S-shape-only kernels keep every tour in its thread: no long-tour pass
     if (p.n_tours > 0 && !wh::sshape_kernel_applies(a)) {

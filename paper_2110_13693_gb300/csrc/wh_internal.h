@@ -66,6 +66,9 @@ struct EvalArgs {
     // k_prep (flags: 1 invalid line, 2 has lines, 4 invalid offsets); NULL
     // otherwise
     uint4* order_agg;
+    // one CTA per plan (k_eval_plan): order << 8 | place in it of every line,
+    // all ones for a line of no order, built by k_prep; NULL otherwise
+    uint32_t* line_ord;
 };
 
 // A work item of the batched launch: 32-tour chunks [chunk_begin, chunk_end)
@@ -338,6 +341,9 @@ cudaError_t launch_prep_batch(const BatchArgs& b, int max_work, cudaStream_t s);
 // routing mask S-shape only on a layout of at most 2,048 aisles: the
 // sort-free S-shape kernel scores the short-tour pass (and every tour)
 bool sshape_kernel_applies(const EvalArgs& a);
+// one CTA per plan (k_eval_plan.cu) instead of one tour per thread (launch_eval_short)
+bool eval_plan_applies(const EvalArgs& a, int num_sms);
+cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_eval_short(const EvalArgs& a, const Tuning& t, int num_sms, cudaStream_t s,
                               int* grid_out);
 cudaError_t launch_eval_batch(const BatchArgs& b, const Tuning& t, bool k16, int num_sms, cudaStream_t s);
