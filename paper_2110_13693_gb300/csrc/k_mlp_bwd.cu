@@ -52,24 +52,43 @@ __device__ __forceinline__ void write_transposed(const __nv_bfloat16 (*s_t)[BT_R
     }
 }
 
+// blockIdx.y: 0 the gradients at the output (dy, loss, dZ2 and its transpose,
+// column sums), 1 the transpose of H1, 2 of X.  The three read nothing of each
+// other, so they are blocks of their own (one after another in a block they
+// took 27 us at 4,096 rows, latency of 128 blocks of three serial passes).
 __global__ void __launch_bounds__(BT_THREADS) k_bwd_tail(BwdArgs b) {
     __shared__ float s_dy[BT_ROWS];
     __shared__ __align__(16) __nv_bfloat16 s_t[256][BT_ROWS + 8];
     const int tid = threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * BT_ROWS;
-    float* part = b.part_t + (int64_t)blockIdx.x * BT_PART;
-    // H1 transposed (the forward's activations; rows past n are zero)
-    {
+    if (blockIdx.y == 1) {
+        // H1 transposed (the forward's activations; rows past n are zero)
         const int j = tid;
-#pragma unroll 8
+#pragma unroll 16
         for (int rr = 0; rr < BT_ROWS; ++rr) {
             const int64_t r = r0 + rr;
             s_t[j][rr] = r < b.n ? b.H1[r * 256 + j] : __float2bfloat16_rn(0.0f);
         }
+        __syncthreads();
+        write_transposed(s_t, 256, b.H1T, b.ldt, r0, tid);
+        return;
     }
-    __syncthreads();
-    write_transposed(s_t, 256, b.H1T, b.ldt, r0, tid);
-    __syncthreads();
+    if (blockIdx.y == 2) {
+        // X transposed, with row 192 = 1 for every row of the batch
+        if (tid <= (int)MLP_IN) {
+#pragma unroll 16
+            for (int rr = 0; rr < BT_ROWS; ++rr) {
+                const int64_t r = r0 + rr;
+                __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
+                if (r < b.n) v = tid < (int)MLP_IN ? b.X[r * MLP_IN + tid] : __float2bfloat16_rn(1.0f);
+                s_t[tid][rr] = v;
+            }
+        }
+        __syncthreads();
+        write_transposed(s_t, (int)MLP_IN + 1, b.XT, b.ldt, r0, tid);
+        return;
+    }
+    float* part = b.part_t + (int64_t)blockIdx.x * BT_PART;
     if (tid < 32) {
         const int64_t r = r0 + tid;
         float d = 0.0f, l = 0.0f;
@@ -123,19 +142,6 @@ __global__ void __launch_bounds__(BT_THREADS) k_bwd_tail(BwdArgs b) {
     }
     __syncthreads();
     write_transposed(s_t, 256, b.dZ2T, b.ldt, r0, tid);
-    __syncthreads();
-    // X transposed, with row 192 = 1 for every row of the batch
-    if (tid <= (int)MLP_IN) {
-#pragma unroll 8
-        for (int rr = 0; rr < BT_ROWS; ++rr) {
-            const int64_t r = r0 + rr;
-            __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
-            if (r < b.n) v = tid < (int)MLP_IN ? b.X[r * MLP_IN + tid] : __float2bfloat16_rn(1.0f);
-            s_t[tid][rr] = v;
-        }
-    }
-    __syncthreads();
-    write_transposed(s_t, (int)MLP_IN + 1, b.XT, b.ldt, r0, tid);
 }
 
 // ------------------------------------------------------------------- dZ1
@@ -147,7 +153,13 @@ constexpr int D1_NBARS = 6;   // w_full, a_full, a_empty, acc_full, acc_empty, d
 constexpr uint32_t D1_OFF_MISC = D1_OFF_BAR + 8 * D1_NBARS;
 constexpr uint32_t D1_SMEM = D1_OFF_MISC + 16 + 1024;
 
-__global__ void __launch_bounds__(BW_THREADS, 1)
+// 16 epilogue warps, four per TMEM lane quarter with 64 columns each: the
+// epilogue is gelu' (erff and expf) of every element, which four warps on one
+// of four schedulers each took 28 us for at 4,096 rows.
+constexpr int D1_EPI_WARPS = 16;
+constexpr int D1_THREADS = (BW_EPI0 + D1_EPI_WARPS) * 32;
+
+__global__ void __launch_bounds__(D1_THREADS, 1)
     k_mlp_dz1(const __grid_constant__ CUtensorMap mdz2, const __grid_constant__ CUtensorMap mw2, BwdArgs b) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -166,7 +178,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         mbar_init(a_full, 1);
         mbar_init(a_empty, 1);
         mbar_init(acc_full, 1);
-        mbar_init(acc_empty, 128);
+        mbar_init(acc_empty, D1_EPI_WARPS * 32);
         mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -219,34 +231,38 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
             mbar_drain(done, 0);
         }
     } else {
-        const int quarter = warp & 3;
+        const int quarter = warp & 3, part_id = (warp - BW_EPI0) >> 2;
         const int r = 32 * quarter + lane;
         const uint32_t lane_addr = (uint32_t)(32 * quarter) << 16;
         uint32_t it = 0;
         for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
-            if (!__all_sync(0xffffffffu, mbar_wait(acc_full, it & 1u, abort, b.status))) break;
-            tc_fence_after();
             const int64_t row = tile * 128 + r;
             const bool live = row < b.n;
+            if (!__all_sync(0xffffffffu, mbar_wait(acc_full, it & 1u, abort, b.status))) break;
+            tc_fence_after();
 #pragma unroll 1
-            for (int cc = 0; cc < 8; ++cc) {
-                float v[32];
-                tc_ld32(tmem + lane_addr + (uint32_t)(32 * cc), v);
-                if (!live) continue;
-                const float* z = b.Z1 + row * 256 + 32 * cc;
+            for (int cc = 0; cc < 4; ++cc) {
+                const int col = 64 * part_id + 16 * cc;
+                float v[16];
+                tc_ld16(tmem + lane_addr + (uint32_t)col, v);
+                if (live) {
+                    uint32_t h[8];
 #pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    const float4 za = *reinterpret_cast<const float4*>(z + 8 * g8);
-                    const float4 zb = *reinterpret_cast<const float4*>(z + 8 * g8 + 4);
-                    const float zz[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
-                    __nv_bfloat16 h[8];
+                    for (int g8 = 0; g8 < 2; ++g8) {
+                        float zz[8];
+                        ld_global_32b(b.Z1 + row * 256 + col + 8 * g8, zz);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) h[e] = __float2bfloat16_rn(v[8 * g8 + e] * gelu_grad(zz[e]));
-                    const int col = 32 * cc + 8 * g8;
-                    *reinterpret_cast<uint4*>(b.dZ1 + row * 256 + col) = *reinterpret_cast<const uint4*>(h);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) b.dZ1T[(int64_t)(col + e) * b.ldt + row] = h[e];
+                        for (int e = 0; e < 8; e += 2) {
+                            const __nv_bfloat16 h0 = __float2bfloat16_rn(v[8 * g8 + e] * gelu_grad(zz[e]));
+                            const __nv_bfloat16 h1 = __float2bfloat16_rn(v[8 * g8 + e + 1] * gelu_grad(zz[e + 1]));
+                            b.dZ1T[(int64_t)(col + 8 * g8 + e) * b.ldt + row] = h0;
+                            b.dZ1T[(int64_t)(col + 8 * g8 + e + 1) * b.ldt + row] = h1;
+                            h[4 * g8 + e / 2] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                        }
+                    }
+                    st_global_32b(b.dZ1 + row * 256 + col, h);
                 }
+                __syncwarp();
             }
             tc_fence_before();
             mbar_arrive(acc_empty);
@@ -379,36 +395,41 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
 }
 
 // ------------------------------------------------------------------- Adam
+// p[0] + p[step] + ... (count terms) added in this order, 16 loads in flight
+__device__ __forceinline__ float sum_parts(const float* p, int64_t step, int count) {
+    float acc = 0.0f;
+    for (int k0 = 0; k0 < count; k0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = k0 + u < count ? p[(int64_t)(k0 + u) * step] : 0.0f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+            if (k0 + u < count) acc += v[u];
+    }
+    return acc;
+}
+
 // Every gradient the sum of its partials in a fixed order, written to G, then
 // one Adam step on the fp32 master parameters; the bf16 copies of w1 and w2
-// follow.  Block 0 also sums the loss.
+// follow, row-major and transposed (what the next forward's tensor maps
+// describe).  Block 0 also sums the loss.
 __global__ void k_adam_parts(BwdArgs b, float* p, float* mo, float* ve, float* G, float lr, float b1, float b2,
-                             float eps, float c1, float c2, __nv_bfloat16* w1b, __nv_bfloat16* w2b, float* loss) {
+                             float eps, float c1, float c2, __nv_bfloat16* w1b, __nv_bfloat16* w2b,
+                             __nv_bfloat16* w1t, __nv_bfloat16* w2t, float* loss) {
     const int S = b.splits;
     const int nbt = (int)((b.n + BT_ROWS - 1) / BT_ROWS);
     const float* pw2 = b.part_w;                            // [S][256][256]
     const float* pw1 = b.part_w + (int64_t)S * 65536;       // [S][256][256], row 192 = b1
-    if (blockIdx.x == 0 && threadIdx.x == 0 && loss) {
-        float l = 0.0f;
-        for (int k = 0; k < nbt; ++k) l += b.part_t[(int64_t)k * BT_PART + 513];
-        *loss = l;
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && loss) *loss = sum_parts(b.part_t + 513, BT_PART, nbt);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < MLP_NPARAM;
          i += (int64_t)gridDim.x * blockDim.x) {
-        float gi = 0.0f;
-        if (i < MLP_W1) {
-            for (int s = 0; s < S; ++s) gi += pw1[(int64_t)s * 65536 + i];
-        } else if (i < MLP_W2_OFF) {
-            for (int s = 0; s < S; ++s) gi += pw1[(int64_t)s * 65536 + 192 * 256 + (i - MLP_B1_OFF)];
-        } else if (i < MLP_B2_OFF) {
-            for (int s = 0; s < S; ++s) gi += pw2[(int64_t)s * 65536 + (i - MLP_W2_OFF)];
-        } else if (i < MLP_W3_OFF) {
-            for (int k = 0; k < nbt; ++k) gi += b.part_t[(int64_t)k * BT_PART + (i - MLP_B2_OFF)];
-        } else if (i < MLP_B3_OFF) {
-            for (int k = 0; k < nbt; ++k) gi += b.part_t[(int64_t)k * BT_PART + 256 + (i - MLP_W3_OFF)];
-        } else {
-            for (int k = 0; k < nbt; ++k) gi += b.part_t[(int64_t)k * BT_PART + 512];
-        }
+        float gi;
+        if (i < MLP_W1) gi = sum_parts(pw1 + i, 65536, S);
+        else if (i < MLP_W2_OFF) gi = sum_parts(pw1 + 192 * 256 + (i - MLP_B1_OFF), 65536, S);
+        else if (i < MLP_B2_OFF) gi = sum_parts(pw2 + (i - MLP_W2_OFF), 65536, S);
+        else if (i < MLP_W3_OFF) gi = sum_parts(b.part_t + (i - MLP_B2_OFF), BT_PART, nbt);
+        else if (i < MLP_B3_OFF) gi = sum_parts(b.part_t + 256 + (i - MLP_W3_OFF), BT_PART, nbt);
+        else gi = sum_parts(b.part_t + 512, BT_PART, nbt);
         G[i] = gi;
         const float mi = b1 * mo[i] + (1.0f - b1) * gi;
         const float vi = b2 * ve[i] + (1.0f - b2) * gi * gi;
@@ -416,8 +437,15 @@ __global__ void k_adam_parts(BwdArgs b, float* p, float* mo, float* ve, float* G
         ve[i] = vi;
         const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
         p[i] = pi;
-        if (i < MLP_W1) w1b[i] = __float2bfloat16_rn(pi);
-        else if (i >= MLP_W2_OFF && i < MLP_W2_OFF + MLP_W2) w2b[i - MLP_W2_OFF] = __float2bfloat16_rn(pi);
+        const __nv_bfloat16 h = __float2bfloat16_rn(pi);
+        if (i < MLP_W1) {
+            w1b[i] = h;
+            w1t[(i & 255) * MLP_IN + (i >> 8)] = h;
+        } else if (i >= MLP_W2_OFF && i < MLP_W2_OFF + MLP_W2) {
+            const int64_t k = i - MLP_W2_OFF;
+            w2b[k] = h;
+            w2t[(k & 255) * 256 + (k >> 8)] = h;
+        }
     }
 }
 
@@ -430,13 +458,13 @@ cudaError_t launch_bwd(const BwdArgs& b, const CUtensorMap& mdz2, const CUtensor
                        cudaStream_t s) {
     if (b.n <= 0) return cudaSuccess;
     const int64_t nbt = (b.n + BT_ROWS - 1) / BT_ROWS;
-    k_bwd_tail<<<(unsigned)nbt, BT_THREADS, 0, s>>>(b);
+    k_bwd_tail<<<dim3((unsigned)nbt, 3), BT_THREADS, 0, s>>>(b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_mlp_dz1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (b.n + 127) / 128;
-    k_mlp_dz1<<<(unsigned)(tiles < num_sms ? tiles : num_sms), BW_THREADS, D1_SMEM, s>>>(mdz2, mw2, b);
+    k_mlp_dz1<<<(unsigned)(tiles < num_sms ? tiles : num_sms), D1_THREADS, D1_SMEM, s>>>(mdz2, mw2, b);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM);
@@ -446,12 +474,13 @@ cudaError_t launch_bwd(const BwdArgs& b, const CUtensorMap& mdz2, const CUtensor
 }
 
 cudaError_t launch_adam_parts(const BwdArgs& b, float* p, float* m, float* v, float* G, float lr, int step, void* w1b,
-                              void* w2b, float* loss, cudaStream_t s) {
+                              void* w2b, void* w1t, void* w2t, float* loss, cudaStream_t s) {
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
     const int blocks = (int)((MLP_NPARAM + 255) / 256);
     k_adam_parts<<<blocks, 256, 0, s>>>(b, p, m, v, G, lr, b1, b2, 1e-8f, c1, c2, static_cast<__nv_bfloat16*>(w1b),
-                                        static_cast<__nv_bfloat16*>(w2b), loss);
+                                        static_cast<__nv_bfloat16*>(w2b), static_cast<__nv_bfloat16*>(w1t),
+                                        static_cast<__nv_bfloat16*>(w2t), loss);
     return cudaGetLastError();
 }
 

@@ -221,24 +221,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             // computed
             auto e1_chunk = [&](int kc, const uint32_t (&v)[16]) {
                 const int c0 = 64 * kc + 16 * part_id;
+                uint32_t hw[8];
 #pragma unroll
                 for (int g8 = 0; g8 < 2; ++g8) {
                     const int c = c0 + 8 * g8;
                     const ulonglong2 bA = *reinterpret_cast<const ulonglong2*>(par + c);
                     const ulonglong2 bB = *reinterpret_cast<const ulonglong2*>(par + c + 4);
                     const uint64_t bias[4] = {bA.x, bA.y, bB.x, bB.y};
-                    uint32_t w[4];
+                    uint64_t z[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const uint64_t z = add2(pk(__uint_as_float(v[8 * g8 + 2 * j]),
-                                                   __uint_as_float(v[8 * g8 + 2 * j + 1])), bias[j]);
-                        if (save_rows) *reinterpret_cast<uint64_t*>(save.Z1 + row * 256 + c + 2 * j) = z;
+                        z[j] = add2(pk(__uint_as_float(v[8 * g8 + 2 * j]), __uint_as_float(v[8 * g8 + 2 * j + 1])),
+                                    bias[j]);
                         float g0, g1;
-                        upk(gelu2(z), g0, g1);
-                        w[j] = pack_bf16(g0, g1);
+                        upk(gelu2(z[j]), g0, g1);
+                        hw[4 * g8 + j] = pack_bf16(g0, g1);
                     }
-                    const uint4 o = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (save_rows) *reinterpret_cast<uint4*>(save.H1 + row * 256 + c) = o;
+                    if (save_rows) st_global_32b(save.Z1 + row * 256 + c, z[0], z[1], z[2], z[3]);
+                    const uint4 o = make_uint4(hw[4 * g8], hw[4 * g8 + 1], hw[4 * g8 + 2], hw[4 * g8 + 3]);
                     // 128-byte swizzle: 16-byte chunk j of row r sits at chunk j ^ (r % 8)
                     const int chunk = (c & 63) >> 3;
                     unsigned char* dst = smem + OFF_H + (c >> 6) * ATOM + r * 128 + ((chunk ^ (r & 7)) << 4);
@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tc_fence_before();
                 mbar_arrive(h1c(kc));
+                if (save_rows) st_global_32b(save.H1 + row * 256 + c0, hw);
             };
             uint32_t ta[16], tb[16];
             tc_ld16_issue(tmem + lane_addr + (uint32_t)(16 * part_id), ta);
@@ -265,6 +266,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             // next step's TMEM load in flight while one is computed
             uint64_t part2 = dup2(0.0f);
             auto e2_step = [&](int c0, const uint32_t (&v)[16]) {
+                uint32_t hw[8];
+                uint64_t zs[4];
 #pragma unroll
                 for (int j4 = 0; j4 < 16; j4 += 4) {
                     const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(par + 256 + c0 + j4);
@@ -277,14 +280,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         upk(gelu2(z), g0, g1);
                         // the layer-2 activations are bf16 values
                         const uint32_t hb = pack_bf16(g0, g1);
-                        if (save_rows) {
-                            *reinterpret_cast<uint64_t*>(save.Z2 + row * 256 + c0 + j) = z;
-                            *reinterpret_cast<uint32_t*>(save.H2 + row * 256 + c0 + j) = hb;
-                        }
+                        hw[j / 2] = hb;
+                        zs[j / 2 % 4] = z;
+                        if (save_rows && j % 8 == 6)
+                            st_global_32b(save.Z2 + row * 256 + c0 + j - 6, zs[0], zs[1], zs[2], zs[3]);
                         const uint64_t hv = pk(__uint_as_float(hb << 16), __uint_as_float(hb & 0xFFFF0000u));
                         part2 = fma2(hv, h ? w3.y : w3.x, part2);
                     }
                 }
+                if (save_rows) st_global_32b(save.H2 + row * 256 + c0, hw);
             };
             const uint32_t c2 = (uint32_t)(TC_PART_COLS * part_id);
             tc_ld16_issue(tmem + lane_addr + 256u + c2, ta);

@@ -172,6 +172,26 @@ __device__ __forceinline__ void tc_wait_ld16(uint32_t (&r)[16]) {
                  : "memory");
 }
 
+// 32 bytes of a row to / from global memory in one access (32-byte aligned):
+// a lane's own row is a sector of its own, so a warp's access moves 32 full
+// sectors instead of 32 parts of them four or eight times over.
+__device__ __forceinline__ void st_global_32b(void* p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_global_32b(void* p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
+    asm volatile("st.global.v4.b64 [%0], {%1,%2,%3,%4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+
+__device__ __forceinline__ void ld_global_32b(const void* p, float (&v)[8]) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+
 // Pairs of fp32 values in one 64-bit register for the packed fp32x2
 // arithmetic of sm_100 and later (add / mul / fma .f32x2, element-wise,
 // round to nearest): the epilogue's FMA-pipe work in half the instructions.

@@ -299,7 +299,7 @@ cudaError_t launch_bwd(const BwdArgs& b, const CUtensorMap& mdz2, const CUtensor
                        const CUtensorMap& mdz2t, const CUtensorMap& mxt, const CUtensorMap& mdz1t, int num_sms,
                        cudaStream_t s);
 cudaError_t launch_adam_parts(const BwdArgs& b, float* p, float* m, float* v, float* G, float lr, int step, void* w1b,
-                              void* w2b, float* loss, cudaStream_t s);
+                              void* w2b, void* w1t, void* w2t, float* loss, cudaStream_t s);
 
 struct FeatConst {
     int32_t A, L;

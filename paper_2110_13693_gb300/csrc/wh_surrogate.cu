@@ -331,9 +331,9 @@ extern "C" int wh_surrogate_train_step(wh_surrogate* s, const uint16_t* X, const
     if (wh::launch_bwd(b, mdz2, s->mw2r, mh1t, mdz2t, mxt, mdz1t, s->num_sms, st) != cudaSuccess) return WH_ECUDA;
     s->last_n = n;
     s->step += 1;
-    if (wh::launch_adam_parts(b, s->P, s->Mo, s->Ve, s->G, lr, s->step, s->w1b, s->w2b, s->loss, st) != cudaSuccess)
+    if (wh::launch_adam_parts(b, s->P, s->Mo, s->Ve, s->G, lr, s->step, s->w1b, s->w2b, s->w1t, s->w2t, s->loss,
+                              st) != cudaSuccess)
         return WH_ECUDA;
-    s->t_stale = true;
     if (loss_out && cudaMemcpyAsync(loss_out, s->loss, sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return WH_ECUDA;
     return WH_OK;
