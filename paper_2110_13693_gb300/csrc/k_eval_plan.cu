@@ -16,20 +16,16 @@
 //   cost       a thread per tour, ordered by line count: one pass over the
 //              sorted row, a DP step where an aisle ends (no record slots,
 //              so no limit on a tour's aisles).
-#include "tour_core.cuh"
+#include "row_core.cuh"
 
 namespace wh {
 namespace {
 
 constexpr int PL_THREADS = 256;
 constexpr int PL_CTAS = 3;       // per SM
-constexpr int PL_MAXN = 128;     // lines of a tour (8 lanes of 16); longer ones go to the long-tour pass
+constexpr int PL_MAXN = ROW_MAXN;   // longer tours go to the long-tour pass
 constexpr int PL_LIST = 1024;    // tours of a plan taken per round
 constexpr int PL_U = PL_LIST / PL_THREADS;
-
-// Markers of unusable lines (a key's aisle is at most 65,533, so both compare
-// above every key); KEY_BAD: location out of range.
-constexpr uint32_t KEY_BAD_SKU = 0xFFFFFFFDu;
 
 // Line count of tour t, its orders checked: -1 for invalid offsets or ids
 // (flagged), PL_MAXN + 1 for a tour that the long-tour pass takes.  Four
@@ -59,59 +55,6 @@ __device__ __forceinline__ int count_lines(const EvalArgs& a, const uint8_t* s_c
         return -1;
     }
     return n;
-}
-
-// Sort the rows of tours list[i0 + lane / G] (those below i1), G lanes a tour
-// with 16 keys each.
-template <int G>
-__device__ __forceinline__ void sort_rows(uint32_t* rows, const uint16_t* s_list, const uint16_t* s_base,
-                                          const uint8_t* s_n, int i0, int i1, int lane) {
-    const int sub = lane & (G - 1), i = i0 + lane / G;
-    int n = 0;
-    uint32_t* row = rows;
-    if (i < i1) {
-        const int k = s_list[i];
-        n = s_n[k];
-        row = rows + s_base[k];
-    }
-    uint32_t x[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) x[j] = j * G + sub < n ? row[j * G + sub] : KEY_NONE;
-    merge_exchange<16>(x);
-#pragma unroll
-    for (int s = 1; s < G; s <<= 1) {
-        // blocks of s lanes merged in pairs: every key against its mirror
-        const bool low = (lane & s) == 0;
-        uint32_t y[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) y[j] = __shfl_xor_sync(0xffffffffu, x[15 - j], 2 * s - 1);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) x[j] = low ? min(x[j], y[j]) : max(x[j], y[j]);
-#pragma unroll
-        for (int d = s >> 1; d > 0; d >>= 1) {
-            const bool l2 = (lane & d) == 0;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const uint32_t o = __shfl_xor_sync(0xffffffffu, x[j], d);
-                x[j] = l2 ? min(x[j], o) : max(x[j], o);
-            }
-        }
-#pragma unroll
-        for (int d = 8; d > 0; d >>= 1) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                if ((j ^ d) > j) {
-                    const uint32_t p = x[j], r = x[j ^ d];
-                    x[j] = min(p, r);
-                    x[j ^ d] = max(p, r);
-                }
-            }
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-        if (sub * 16 + j < n) row[sub * 16 + j] = x[j];
 }
 
 // sum over the warp's lanes of values 0 <= v < 2^31
@@ -283,9 +226,9 @@ __global__ void __launch_bounds__(PL_THREADS, PL_CTAS) k_eval_plan(EvalArgs a) {
                 int u = lane == 0 ? atomicAdd(&s_unit, 1) : 0;
                 u = __shfl_sync(0xffffffffu, u, 0);
                 if (u >= un) break;
-                if (u < u8n) sort_rows<8>(rows, s_list, s_base, s_n, 4 * u, c8, lane);
-                else if (u < u4n) sort_rows<4>(rows, s_list, s_base, s_n, c8 + 8 * (u - u8n), c4, lane);
-                else sort_rows<2>(rows, s_list, s_base, s_n, c4 + 16 * (u - u4n), total, lane);
+                const int G = u < u8n ? 8 : u < u4n ? 4 : 2;
+                const int i0 = G == 8 ? 4 * u : G == 4 ? c8 + 8 * (u - u8n) : c4 + 16 * (u - u4n);
+                sort_rows(G, rows, s_list, s_base, s_n, i0, G == 8 ? c8 : G == 4 ? c4 : total, lane);
             }
             __syncthreads();
             // ---- cost
@@ -294,35 +237,9 @@ __global__ void __launch_bounds__(PL_THREADS, PL_CTAS) k_eval_plan(EvalArgs a) {
                 const bool on = i0 + lane < total;
                 const int k = on ? s_list[i0 + lane] : 0, t = tb + k, n = on ? s_n[k] : 0;
                 const uint32_t* row = rows + (on ? s_base[k] : 0);
-                DP5 v;
-                dp_init(v);
-                int pa = 0, m = 0;
-                uint32_t key = n > 0 ? row[0] : 0u, lo = key, gi = 0, last = 0;
-                for (int p = 0; p < n; p += 4) {
-                    uint32_t nx[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) nx[j] = p + j + 1 < n ? row[p + j + 1] : KEY_NONE;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (nx[j] > (key | 0xFFFFu)) {
-                            const int ai = (int)(key >> 16);
-                            if (need_rr)
-                                dp_aisle_rel(v, c, ai - pa, (int)(lo & 0xFFFFu), (int)(key & 0xFFFFu), (int)gi);
-                            pa = ai;
-                            ++m;
-                            last = key;
-                            lo = nx[j];
-                            gi = 0;
-                        } else {
-                            gi = max(gi, nx[j] - key);
-                        }
-                        key = nx[j];
-                    }
-                }
-                // markers sort last and never end an aisle
+                int cs, cr;
+                row_costs(a.g, c, row, n, need_rr, cs, cr);
                 const bool kbad = n > 0 && row[n - 1] >= KEY_BAD_SKU;
-                const int cs = sshape_cost(a.g, m, (int)(last >> 16), (int)(last & 0xFFFFu));
-                const int cr = need_rr ? dp_final(v) + c.p2 * pa : 0;
                 if (kbad) {
                     if constexpr (!SHARED_MAP)   // under a shared slotting k_prep has flagged the line
                         for (int p = n - 1; p >= 0 && row[p] >= KEY_BAD_SKU; --p)

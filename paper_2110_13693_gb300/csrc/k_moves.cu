@@ -11,12 +11,12 @@
 //                              locations exchanged.
 // Pipeline: per-tour line counts and the plan's order -> tour map; the SKU ->
 // orders index of the order book; per move a check, a status and a task count;
-// an exclusive scan of the counts; the task list; one task per thread (tasks
-// over SHORT_MAX lines: one warp each) re-costing one changed tour and adding
+// an exclusive scan of the counts; the task list; a warp per 32 tasks (one for
+// each task over ROW_MAXN lines) re-costing the changed tours and adding
 // (new - old) into the move's two int64 deltas.  A SKU-swap move lists one task
 // per (order with s1 or s2); of the tasks that land in the same tour only the
 // one of the smallest such order counts, so no de-duplication pass is needed.
-#include "tour_core.cuh"
+#include "row_core.cuh"
 #include "feat_core.cuh"
 
 namespace wh {
@@ -97,17 +97,27 @@ __global__ void __launch_bounds__(MVT_THREADS) k_mv_tours_plan(MoveArgs M) {
                 flag(a.status, WH_STATUS_BAD_OFFSET);
                 lines = -1;
             } else {
-                for (int q = q0; q < q1; ++q) {
-                    const int o = a.order_seq[q];
-                    int lb, le;
-                    const int c = order_lines_checked(a, o, lb, le);
-                    if (c < 0) {
-                        flag(a.status, WH_STATUS_BAD_ORDER);
-                        lines = -1;
-                        break;
+                // four orders' ids, then their line ranges, in flight
+                for (int q = q0; q < q1 && lines >= 0; q += 4) {
+                    int o[4], cnt[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) o[u] = q + u < q1 ? a.order_seq[q + u] : 0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        int lb, le;
+                        cnt[u] = q + u < q1 ? order_lines_checked(a, o[u], lb, le) : 0;
                     }
-                    lines += c;
-                    s_row[o] = t;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (q + u >= q1 || lines < 0) continue;
+                        if (cnt[u] < 0) {
+                            flag(a.status, WH_STATUS_BAD_ORDER);
+                            lines = -1;
+                        } else {
+                            lines += cnt[u];
+                            s_row[o[u]] = t;
+                        }
+                    }
                 }
             }
             M.tour_lines[t] = lines;
@@ -127,41 +137,58 @@ __global__ void k_mv_sku_count(MoveArgs M) {
     }
 }
 
-// one block: exclusive scan of the per-SKU counts into sku_off, cursors reset
-__global__ void k_mv_sku_scan(MoveArgs M) {
+// one block: exclusive scan of the per-SKU counts into sku_off, cursors
+// reset.  16 SKUs a thread and round, read and written 16 bytes at a time:
+// 50,000 SKUs in four rounds (one SKU a thread took 49 rounds, 49 us).
+constexpr int SKU_SCAN_T = 1024, SKU_SCAN_V = 16;
+
+__global__ void __launch_bounds__(SKU_SCAN_T) k_mv_sku_scan(MoveArgs M) {
     __shared__ int warp_tot[32];
-    __shared__ int carry;
     const int n = M.a.n_sku, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (tid == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += blockDim.x) {
-        const int i = base + tid;
-        const int v = i < n ? M.sku_cur[i] : 0;
-        int x = v;
+    int carry = 0;
+    for (int base = 0; base < n; base += SKU_SCAN_T * SKU_SCAN_V) {
+        const int i0 = base + tid * SKU_SCAN_V;
+        int v[SKU_SCAN_V], sum = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += u;
-        }
-        if (lane == 31) warp_tot[w] = x;
-        __syncthreads();
-        if (w == 0) {
-            int y = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, y, o);
-                if (lane >= o) y += u;
+        for (int u = 0; u < SKU_SCAN_V; u += 4) {
+            int4 x = make_int4(0, 0, 0, 0);
+            if (i0 + u + 4 <= n) x = *reinterpret_cast<const int4*>(M.sku_cur + i0 + u);
+            else {
+                if (i0 + u < n) x.x = M.sku_cur[i0 + u];
+                if (i0 + u + 1 < n) x.y = M.sku_cur[i0 + u + 1];
+                if (i0 + u + 2 < n) x.z = M.sku_cur[i0 + u + 2];
             }
-            warp_tot[lane] = y;
+            v[u] = x.x;
+            v[u + 1] = x.y;
+            v[u + 2] = x.z;
+            v[u + 3] = x.w;
         }
+#pragma unroll
+        for (int u = 0; u < SKU_SCAN_V; ++u) sum += v[u];
+        const int incl = warp_inclusive_scan(sum);
+        if (lane == 31) warp_tot[w] = incl;
         __syncthreads();
-        const int excl = carry + (w ? warp_tot[w - 1] : 0) + x - v;
-        if (i < n) {
-            M.sku_off[i] = excl;
-            M.sku_cur[i] = 0;
+        const int t = warp_tot[lane];
+        const int tot = warp_inclusive_scan(t);
+        int e = carry + incl - sum + __shfl_sync(0xffffffffu, tot - t, w);
+        carry += __shfl_sync(0xffffffffu, tot, 31);
+#pragma unroll
+        for (int u = 0; u < SKU_SCAN_V; u += 4) {
+            const int4 x = make_int4(e, e + v[u], e + v[u] + v[u + 1], e + v[u] + v[u + 1] + v[u + 2]);
+            e = x.w + v[u + 3];
+            if (i0 + u + 4 <= n) {
+                *reinterpret_cast<int4*>(M.sku_off + i0 + u) = x;
+                *reinterpret_cast<int4*>(M.sku_cur + i0 + u) = make_int4(0, 0, 0, 0);
+            } else {
+                const int xs[3] = {x.x, x.y, x.z};
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    if (i0 + u + k >= n) continue;
+                    M.sku_off[i0 + u + k] = xs[k];
+                    M.sku_cur[i0 + u + k] = 0;
+                }
+            }
         }
-        __syncthreads();
-        if (tid == blockDim.x - 1) carry = excl + v;
         __syncthreads();
     }
     if (tid == 0) M.sku_off[n] = carry;
@@ -390,147 +417,272 @@ __device__ __forceinline__ int task_loc(const int32_t* map, int s, const int4 mv
 // the line's SKU is one the SKU move changes
 __device__ __forceinline__ bool sku_hit(int s, const int4 mv) { return s == mv.y || (mv.x == 2 && s == mv.z); }
 
-// Walk the changed tour of task `tk`: calls emit(key) for every line, in
-// order; returns false on an invalid id.  For SKU-swap tasks also reports
-// whether the task is the counted one of its tour.
-template <typename Emit>
-__device__ __forceinline__ bool walk_task(const MoveArgs& M, const int4 tk, const int4 mv, bool& primary,
-                                          Emit emit) {
-    const EvalArgs& a = M.a;
-    const bool swap = mv.x >= 2;   // SKU moves: swap or relocation
-    const int32_t* map = a.slot_map + (int64_t)mv.w * a.slot_stride;
-    const int q0 = a.tour_off[tk.y], q1 = a.tour_off[tk.y + 1];
-    const int add = (!swap && tk.z >= 0) ? tk.z : -1;
-    const int rem = (!swap && tk.w >= 0) ? tk.w : -1;
-    int hit_min = 0x7fffffff;
-    bool own_has_s1 = false;
-    bool ok = q0 >= 0 && q1 >= q0 && (int64_t)q1 <= a.n_seq;
-    // the orders walked: positions q0..q1-1 of order_seq (without `rem`),
-    // then the added order; ids two ahead and line bounds one ahead are in
-    // flight while the current order's lines are gathered
-    const int q_end = !ok ? q0 : (add >= 0 ? q1 + 1 : q1);
-    auto order_at = [&](int q) { return q < q1 ? a.order_seq[q] : add; };
-    int o0 = q0 < q_end ? order_at(q0) : 0;
-    int o1 = q0 + 1 < q_end ? order_at(q0 + 1) : 0;
-    int lb0 = 0, le0 = 0;
-    bool v0 = q0 < q_end && order_lines_checked(a, o0, lb0, le0) >= 0;
-    for (int q = q0; ok && q < q_end; ++q) {
-        const int o = o0;
-        const int lb = lb0, le = le0;
-        const bool valid = v0;
-        const int o2 = q + 2 < q_end ? order_at(q + 2) : 0;
-        v0 = q + 1 < q_end && order_lines_checked(a, o1, lb0, le0) >= 0;
-        o0 = o1;
-        o1 = o2;
-        if (q < q1 && o == rem) continue;
-        if (!valid) { ok = false; break; }
-        // four lines at a time: their SKU loads, then their slot loads (the
-        // plan's own slotting, mostly DRAM), are in flight together
-        for (int l = lb; ok && l < le; l += 4) {
-            int sk[4], loc[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sk[j] = l + j < le ? a.line_sku[l + j] : 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                loc[j] = -1;
-                if (l + j >= le) continue;
-                const int sj = sk[j];
-                if ((unsigned)sj >= (unsigned)a.n_sku) { ok = false; continue; }
-                if (swap && sku_hit(sj, mv)) {
-                    hit_min = min(hit_min, o);
-                    if (o == tk.z && sj == mv.y) own_has_s1 = true;
-                }
-                loc[j] = task_loc(map, sj, mv);
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (!ok || l + j >= le) continue;
-                if ((unsigned)loc[j] >= (unsigned)a.g.n_loc) { ok = false; continue; }
-                emit(loc_key(a.g, loc[j]));
-            }
-        }
-    }
-    primary = !swap || (hit_min == tk.z && (tk.w == -2 || !own_has_s1));
-    return ok;
-}
+// Tasks of at most ROW_MAXN lines: a warp takes 32 tasks, one a lane, and
+// runs them together, as many of one plan at a time as its rows of shared
+// memory hold.  Task by task the lanes take the changed tour's orders (the
+// next task's ids in flight) and put its lines' SKUs, the moved ones already
+// exchanged, into the task's row; then the slot-map gathers of all rows run
+// flat, eight a lane in flight; then the rows are sorted (sort_rows) and each
+// lane costs its own task.  Few registers and no dependent gather per line:
+// 585,000 tasks of 262,144 moves at paper scale (60 lines each) took 505 us
+// one task a thread plus 180 us for the third of them with over 64 lines or
+// 32 aisles.
+constexpr int MV_WARPS = MV_THREADS / 32;
+constexpr int MV_ROWS = 2048;              // keys of a warp's rows: 32 tours of 64 lines
+constexpr uint32_t SKU_BAD = 0x7FFFFFFFu;  // in a row before the gathers: unusable SKU
+constexpr uint32_t SKU_AT = 0x80000000u;   // a relocated SKU: SKU_AT | its location
 
-template <bool KEY16>
-__global__ void __launch_bounds__(MV_THREADS) k_mv_eval(MoveArgs M) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int T = blockDim.x, tid = threadIdx.x, lane = tid & 31;
-    uint32_t* col16 = reinterpret_cast<uint32_t*>(smem) + tid;
-    uint2* col32 = reinterpret_cast<uint2*>(smem) + tid;
+__global__ void __launch_bounds__(MV_THREADS, 5) k_mv_eval(MoveArgs M) {
+    extern __shared__ __align__(16) uint32_t mv_rows[];
+    __shared__ uint16_t s_base[MV_WARPS][32], s_list[MV_WARPS][32];
+    __shared__ uint8_t s_n[MV_WARPS][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    uint32_t* rows = mv_rows + wid * MV_ROWS;
+    uint16_t* bases = s_base[wid];
+    uint16_t* list = s_list[wid];
+    uint8_t* ns = s_n[wid];
     const EvalArgs& a = M.a;
-    const int64_t n_tasks = M.n_tasks;
-    const int64_t warps = (int64_t)gridDim.x * (T >> 5);
-    for (int64_t base = ((int64_t)blockIdx.x * (T >> 5) + (tid >> 5)) * 32; base < n_tasks; base += warps * 32) {
-        const int64_t i = base + lane;
-        const bool active = i < n_tasks;
+    const DPConst c = dp_const(a.g);
+    const int64_t stride = (int64_t)gridDim.x * MV_WARPS * 32;
+    for (int64_t u0 = ((int64_t)blockIdx.x * MV_WARPS + wid) * 32; u0 < M.n_tasks; u0 += stride) {
+        const int64_t i = u0 + lane;
+        const bool active = i < M.n_tasks;
         int4 tk = make_int4(-1, -1, -1, -1), mv = make_int4(0, 0, 0, 0);
-        int n = 0;
-        bool ok = false, primary = false;
         if (active) {
             tk = M.tasks[i];
             mv = M.moves[tk.x];
-            if (tk.y >= 0 && tk.y < a.n_tours) {
-                ok = walk_task(M, tk, mv, primary, [&](uint32_t k) {
-                    if (n < SHORT_MAX) {
-                        if constexpr (KEY16) reinterpret_cast<uint16_t*>(col16 + (n >> 1) * T)[n & 1] = (uint16_t)key16_of(k);
-                        else reinterpret_cast<uint32_t*>(col32 + (n >> 1) * T)[n & 1] = k;
-                    }
-                    ++n;
-                });
-            } else {
-                primary = false;   // an order of the SKU lists outside the plan
-                ok = true;
-            }
-            if (!ok) {
-                flag(a.status, WH_STATUS_BAD_ORDER);
-                M.mstatus[tk.x] = 3;
-            }
         }
-        if (M.stats) {   // changed tours walked and their lines (the moves' roofline)
-            const unsigned walked = __reduce_add_sync(0xffffffffu, active && ok ? 1u : 0u);
-            const unsigned lines = __reduce_add_sync(0xffffffffu, active && ok ? (unsigned)n : 0u);
+        // an order of the SKU lists outside the plan: nothing to cost
+        const bool has = active && tk.y >= 0 && tk.y < a.n_tours;
+        const bool sku_move = mv.x >= 2;
+        bool ok = active;
+        int q0 = 0, q1 = 0, ub = 0;   // ub: the changed tour has at most this many lines
+        const int add = has && !sku_move && tk.z >= 0 ? tk.z : -1;
+        if (has) {
+            q0 = a.tour_off[tk.y];
+            q1 = a.tour_off[tk.y + 1];
+            ub = M.tour_lines[tk.y];
+            int lb, le;
+            const int ca = add >= 0 ? order_lines_checked(a, add, lb, le) : 0;
+            ok = ub >= 0 && ca >= 0;
+            ub = ok ? ub + ca : 0;
+        }
+        const bool lng = has && ok && ub > ROW_MAXN;
+        if (lng) {
+            const int slot = atomicAdd(M.long_count, 1);
+            if (slot < M.long_cap) M.long_list[slot] = (int32_t)i;
+            else { flag(a.status, WH_STATUS_LONG_OVERFLOW); M.mstatus[tk.x] = 3; }
+        }
+        bool run = false;   // the task's cost counts: cs, cr
+        int n = 0, cs = 0, cr = 0;
+        unsigned todo = __ballot_sync(0xffffffffu, has && ok && !lng);
+        while (todo) {
+            // the next tasks of one plan that fit the rows
+            const int plan = __shfl_sync(0xffffffffu, mv.w, __ffs(todo) - 1);
+            const bool cand = ((todo >> lane) & 1u) && mv.w == plan;
+            const int incl = warp_inclusive_scan(cand ? ub : 0);
+            const bool mine = cand && incl <= MV_ROWS;
+            const unsigned take = __ballot_sync(0xffffffffu, mine);
+            const int total = __shfl_sync(0xffffffffu, incl, 31 - __clz(take));
+            todo &= ~take;
+            const int base = mine ? incl - ub : 0;
+            const int32_t* map = a.slot_map + (int64_t)plan * a.slot_stride;
+            bool primary = true;
+            // ids two tasks ahead, line ranges one task ahead
+            int j = __ffs(take) - 1, j2 = j;
+            unsigned left = take & (take - 1);
+            auto first_ids = [&](int k) {
+                const int b0 = __shfl_sync(0xffffffffu, q0, k), b1 = __shfl_sync(0xffffffffu, q1, k);
+                return b0 + lane < b1 ? a.order_seq[b0 + lane] : -1;
+            };
+            int o_cur = first_ids(j), o_nxt = -1;
+            int lb_cur = 0, le_cur = 0;
+            if (o_cur >= 0) {
+                lb_cur = a.order_off[o_cur];
+                le_cur = a.order_off[o_cur + 1];
+            }
+            if (left) {
+                j2 = __ffs(left) - 1;
+                o_nxt = first_ids(j2);
+            }
+            for (;;) {
+                const int b0 = __shfl_sync(0xffffffffu, q0, j), b1 = __shfl_sync(0xffffffffu, q1, j);
+                const int jadd = __shfl_sync(0xffffffffu, add, j), jbase = __shfl_sync(0xffffffffu, base, j);
+                const int type = __shfl_sync(0xffffffffu, mv.x, j);
+                const int mb = __shfl_sync(0xffffffffu, mv.y, j), mc = __shfl_sync(0xffffffffu, mv.z, j);
+                const int tz = __shfl_sync(0xffffffffu, tk.z, j), tw = __shfl_sync(0xffffffffu, tk.w, j);
+                const int jj = j;
+                const bool more = left != 0;
+                int o0 = o_cur, lb0 = lb_cur, le0 = le_cur;   // this lane's order of the first 32
+                j = j2;
+                o_cur = o_nxt;
+                lb_cur = le_cur = 0;
+                if (more) {
+                    if (o_cur >= 0) {
+                        lb_cur = a.order_off[o_cur];
+                        le_cur = a.order_off[o_cur + 1];
+                    }
+                    left &= left - 1;
+                    if (left) {
+                        j2 = __ffs(left) - 1;
+                        o_nxt = first_ids(j2);
+                    }
+                }
+                const bool swap = type >= 2;
+                const int rem = !swap && tw >= 0 ? tw : -1;
+                const int b_end = jadd >= 0 ? b1 + 1 : b1;
+                if (b0 + lane < b1) {
+                    if (o0 == rem) lb0 = le0 = 0;
+                } else if (b0 + lane < b_end) {   // the added order comes last
+                    o0 = jadd;
+                    lb0 = a.order_off[o0];
+                    le0 = a.order_off[o0 + 1];
+                }
+                uint32_t* row = rows + jbase;
+                // the lines' indices at their places (lanes over orders;
+                // ids and line counts were checked with the tour's count)
+                int cnt_all = 0;
+                for (int qb = b0; qb < b_end; qb += 32) {
+                    int lb = lb0, le = le0;
+                    if (qb > b0) {
+                        const int q = qb + lane;
+                        lb = le = 0;
+                        if (q < b_end) {
+                            const int o = q < b1 ? a.order_seq[q] : jadd;
+                            if (!(q < b1 && o == rem)) {
+                                lb = a.order_off[o];
+                                le = a.order_off[o + 1];
+                            }
+                        }
+                    }
+                    const int cnt = le - lb;
+                    const int inc = warp_inclusive_scan(cnt);
+                    uint32_t* w = row + cnt_all + inc - cnt;
+                    for (int l = lb; l < le; ++l) *w++ = (uint32_t)l;
+                    cnt_all += __shfl_sync(0xffffffffu, inc, 31);
+                }
+                __syncwarp();
+                // their SKUs, the move applied: an exchanged SKU takes the
+                // other's place, a relocated one its new location
+                int hit_min = 0x7fffffff;
+                bool own_has_s1 = false;
+                for (int x0 = 0; x0 < cnt_all; x0 += 64) {
+                    int l[2];
+                    uint32_t sk[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int x = x0 + 32 * u + lane;
+                        l[u] = x < cnt_all ? (int)row[x] : -1;
+                        sk[u] = l[u] >= 0 ? (uint32_t)a.line_sku[l[u]] : SKU_BAD;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        uint32_t k = sk[u] < (uint32_t)a.n_sku ? sk[u] : SKU_BAD;
+                        if (swap) {
+                            const bool s1 = k == (uint32_t)mb, hit = s1 || (type == 2 && k == (uint32_t)mc);
+                            // a moved SKU's line: the order that holds it
+                            // (a SKU move keeps every order of the tour)
+                            for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1) {
+                                const int src = __ffs(hits) - 1;
+                                const int hl = __shfl_sync(0xffffffffu, l[u], src);
+                                const bool h1 = __shfl_sync(0xffffffffu, (int)s1, src) != 0;
+                                for (int qb = b0; qb < b1; qb += 32) {
+                                    int o = o0, lb = lb0, le = le0;
+                                    if (qb > b0) {
+                                        lb = le = 0;
+                                        if (qb + lane < b1) {
+                                            o = a.order_seq[qb + lane];
+                                            lb = a.order_off[o];
+                                            le = a.order_off[o + 1];
+                                        }
+                                    }
+                                    if (hl >= lb && hl < le) {
+                                        hit_min = min(hit_min, o);
+                                        own_has_s1 |= h1 && o == tz;
+                                    }
+                                }
+                            }
+                            if (hit) k = type == 3 ? SKU_AT | (uint32_t)mc : (uint32_t)(s1 ? mc : mb);
+                        }
+                        if (l[u] >= 0) row[x0 + 32 * u + lane] = k;
+                    }
+                }
+                if (swap) {
+                    hit_min = __reduce_min_sync(0xffffffffu, hit_min);
+                    own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
+                }
+                if (lane == jj) {
+                    n = cnt_all;
+                    primary = !swap || (hit_min == tz && (tw == -2 || !own_has_s1));
+                }
+                if (!more) break;
+            }
+            __syncwarp();
+            // keys, all rows at once (what lies between rows is translated
+            // too and read by nobody)
+            bool bad = false;
+            for (int x0 = lane; x0 < total; x0 += 256) {
+                uint32_t sk[8];
+                int loc[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) sk[u] = x0 + 32 * u < total ? rows[x0 + 32 * u] : SKU_BAD;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    loc[u] = sk[u] < (uint32_t)a.n_sku ? map[sk[u]] : ((sk[u] & SKU_AT) ? (int)(sk[u] & ~SKU_AT) : -1);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (x0 + 32 * u >= total) continue;
+                    const bool in = (uint32_t)loc[u] < (uint32_t)a.g.n_loc;
+                    bad |= !in;
+                    rows[x0 + 32 * u] = in ? loc_key(a.g, loc[u]) : KEY_BAD;
+                }
+            }
+            bad = __any_sync(0xffffffffu, bad);
+            // sort: the tasks that count, those over 64 lines first
+            const bool cost = mine && primary;
+            const unsigned big = __ballot_sync(0xffffffffu, cost && n > 64), all = __ballot_sync(0xffffffffu, cost);
+            const int n_big = __popc(big), n_all = __popc(all);
+            if (mine) {
+                bases[lane] = (uint16_t)base;
+                ns[lane] = (uint8_t)n;
+            }
+            if (cost) list[n > 64 ? __popc(big & lt_mask) : n_big + __popc(all & ~big & lt_mask)] = (uint16_t)lane;
+            __syncwarp();
+            for (int k = 0; k < n_all;) {
+                const int G = k < n_big ? 8 : 4, end = k < n_big ? n_big : n_all;
+                sort_rows(G, rows, list, bases, ns, k, end, lane);
+                k = min(k + 32 / G, end);
+            }
+            __syncwarp();
+            if (mine) {
+                const uint32_t* row = rows + base;
+                if (cost) row_costs(a.g, c, row, n, true, cs, cr);
+                if (bad)
+                    for (int p = 0; p < n; ++p) ok &= row[p] < KEY_BAD_SKU;
+                run = cost && ok;
+            }
+            __syncwarp();
+        }
+        if (active && !ok) {
+            flag(a.status, WH_STATUS_BAD_ORDER);
+            M.mstatus[tk.x] = 3;
+        }
+        if (M.stats) {   // changed tours walked and their lines (the moves' roofline); k_mv_long_rec adds its own
+            const bool w = active && ok && !lng;
+            const unsigned walked = __reduce_add_sync(0xffffffffu, w ? 1u : 0u);
+            const unsigned lines = __reduce_add_sync(0xffffffffu, w ? (unsigned)n : 0u);
             if (lane == 0 && walked) {
                 atomicAdd(M.stats, (unsigned long long)walked);
                 atomicAdd(M.stats + 1, (unsigned long long)lines);
             }
-        }
-        bool run = active && ok && primary;
-        bool deferred = false;
-        if (run && n > SHORT_MAX) {
-            const int slot = atomicAdd(M.long_count, 1);
-            if (slot < M.long_cap) { M.long_list[slot] = (int32_t)i; deferred = true; }
-            else { flag(a.status, WH_STATUS_LONG_OVERFLOW); M.mstatus[tk.x] = 3; }
-            run = false;
-        }
-        const int nr = run ? n : 0;
-        const int nmax = __reduce_max_sync(0xffffffffu, nr);
-        int cs = 0, cr = 0, m = 0;
-        if constexpr (KEY16) {
-            if (nmax <= 16) tour16<8>(a, col16, T, nr, true, cs, cr, m);
-            else if (nmax <= 32) tour16<16>(a, col16, T, nr, true, cs, cr, m);
-            else tour16<32>(a, col16, T, nr, true, cs, cr, m);
-        } else {
-            if (nmax <= 16) tour32<16>(a, col32, T, nr, true, cs, cr, m);
-            else if (nmax <= 32) tour32<32>(a, col32, T, nr, true, cs, cr, m);
-            else tour32<64>(a, col32, T, nr, true, cs, cr, m);
-        }
-        // more pick aisles than this thread's record slots: the long-task
-        // pass scores the task
-        if (run && m > a.max_rec) {
-            const int slot = atomicAdd(M.long_count, 1);
-            if (slot < M.long_cap) { M.long_list[slot] = (int32_t)i; deferred = true; }
-            else { flag(a.status, WH_STATUS_LONG_OVERFLOW); M.mstatus[tk.x] = 3; }
-            run = false;
         }
         long long ds = 0, dr = 0;
         if (run) {
             ds = (long long)cs - M.tour_s_old[tk.y];
             dr = (long long)cr - M.tour_rr_old[tk.y];
         }
-        if (active && !deferred)   // deferred tasks: k_mv_long writes
+        if (active && !lng)   // k_mv_long_rec and k_mv_long_dp write the long ones
             M.task_cost[i] = run ? make_int2(cs, cr) : make_int2(-1, -1);
         const int key = active ? tk.x : -1;
         const long long ss = segmented_sum(ds, key, lane);
@@ -543,7 +695,7 @@ __global__ void __launch_bounds__(MV_THREADS) k_mv_eval(MoveArgs M) {
     }
 }
 
-// Warp-parallel form of walk_task: lane j takes the changed tour's orders
+// The changed tour of task `tk` by one warp: lane j takes the changed tour's orders
 // j, j + 32, ... (the added order last) and stores their line indices at
 // positions given by a warp prefix sum of the order line counts; then the
 // lanes turn positions x, x + 32, ... into keys.  Only the first `cap`
@@ -623,7 +775,7 @@ __device__ __forceinline__ bool walk_task_warp(const MoveArgs& M, const int4 tk,
     return ok;
 }
 
-// Tasks of more than SHORT_MAX lines, in two kernels.  k_mv_long_rec: one
+// Tasks of more than ROW_MAXN lines, in two kernels.  k_mv_long_rec: one
 // warp per task walks the changed tour (walk_task_warp), sorts its keys in
 // shared memory and extracts the per-aisle records in parallel (a ballot
 // numbers the aisle runs) into a column matrix in global memory; a task with
@@ -642,7 +794,7 @@ __device__ __forceinline__ void mv_long_commit(const MoveArgs& M, int64_t i, int
 __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) {
     __shared__ uint32_t buf[LONG_WARPS][LONG_MAXL];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int count = min(min(*M.long_count, M.long_cap), M.long_rec_cap);
+    const int count = min(*M.long_count, M.long_cap);
     uint32_t* kb = buf[warp];
     const EvalArgs& a = M.a;
     const int64_t cap = M.long_rec_cap;
@@ -654,12 +806,18 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
         bool primary = false;
         const bool ok = walk_task_warp(M, tk, mv, kb, LONG_MAXL, lane, n, primary);
         __syncwarp();
-        if (!ok || n > LONG_MAXL || n < 1) {
+        if (lane == 0 && ok && M.stats) {
+            atomicAdd(M.stats, 1ull);
+            atomicAdd(M.stats + 1, (unsigned long long)n);
+        }
+        if (!ok || n > LONG_MAXL || !primary) {
             if (lane == 0) {
-                flag(a.status, n > LONG_MAXL ? WH_STATUS_TOUR_TOO_LONG : WH_STATUS_BAD_ORDER);
-                M.mstatus[tk.x] = 3;
+                if (!ok || n > LONG_MAXL) {
+                    flag(a.status, n > LONG_MAXL ? WH_STATUS_TOUR_TOO_LONG : WH_STATUS_BAD_ORDER);
+                    M.mstatus[tk.x] = 3;
+                }
                 M.task_cost[i] = make_int2(-1, -1);
-                M.long_m[w] = -1;
+                if (w < cap) M.long_m[w] = -1;
             }
             __syncwarp();
             continue;
@@ -676,7 +834,7 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
             const bool last = in && (x == n - 1 || (int)(kb[x + 1] >> 16) != ai);
             const unsigned fm = __ballot_sync(0xffffffffu, first);
             const int r = m + __popc(fm & ((2u << lane) - 1u)) - 1;
-            if (last && r < MVL_RMAX) {
+            if (last && r < MVL_RMAX && w < cap) {
                 const int hi = (int)(key & 0xFFFFu);
                 int lo = hi, gi = 0;
                 for (int y = x; y > 0 && (int)(kb[y - 1] >> 16) == ai; --y) {
@@ -690,13 +848,14 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
             m += __popc(fm);
         }
         if (lane == 0) {
-            const uint32_t kl = kb[n - 1];   // rightmost aisle, its deepest slot
-            M.long_key[w] = kl;
-            if (m <= MVL_RMAX) {
+            const uint32_t kl = n > 0 ? kb[n - 1] : 0u;   // rightmost aisle, its deepest slot
+            if (m <= MVL_RMAX && w < cap) {
+                M.long_key[w] = kl;
                 M.long_m[w] = m;
             } else {
-                // more aisles than the record matrix keeps: scan and DP here
-                M.long_m[w] = -1;
+                // more aisles, or more tasks, than the record matrix keeps:
+                // scan and DP here
+                if (w < cap) M.long_m[w] = -1;
                 DP5 v;
                 dp_init(v);
                 int pa = 0, lo = 0, prev = 0, gi = 0;
@@ -793,7 +952,7 @@ cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s,
         k_mv_tours<<<grid_of(a.n_tours, 256), 256, 0, s>>>(M);
     }
     if (a.n_lines > 0) k_mv_sku_count<<<grid_of(a.n_lines, 256), 256, 0, s>>>(M);
-    k_mv_sku_scan<<<1, 1024, 0, s>>>(M);
+    k_mv_sku_scan<<<1, SKU_SCAN_T, 0, s>>>(M);
     if (a.n_orders > 0) k_mv_sku_fill<<<grid_of(a.n_orders, 256), 256, 0, s>>>(M);
     k_mv_count<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
     // exclusive scan of n_moves + 1 task counts
@@ -805,31 +964,24 @@ cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s,
     return cudaGetLastError();
 }
 
-size_t moves_eval_smem_bytes(bool k16, int max_rec) {
-    const size_t slots = max_rec > SHORT_MAX / 2 ? (size_t)max_rec : (size_t)(SHORT_MAX / 2);
-    return (k16 ? sizeof(uint32_t) : sizeof(uint2)) * slots * MV_THREADS;
-}
-
 cudaError_t launch_moves_fill(const MoveArgs& M, cudaStream_t s) {
     if (M.n_moves > 0) k_mv_fill<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
     return cudaGetLastError();
 }
 
-cudaError_t launch_moves_eval(const MoveArgs& M, bool k16, int num_sms, cudaStream_t s) {
+cudaError_t launch_moves_eval(const MoveArgs& M, int num_sms, cudaStream_t s) {
     if (M.n_moves > 0) k_mv_fill<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
     if (M.n_tasks > 0) {
-        const size_t smem = moves_eval_smem_bytes(k16, M.a.max_rec);
-        auto kern = k16 ? k_mv_eval<true> : k_mv_eval<false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const size_t smem = sizeof(uint32_t) * MV_ROWS * MV_WARPS;
+        cudaError_t e = cudaFuncSetAttribute(k_mv_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, MV_THREADS, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_eval, MV_THREADS, smem);
         if (e != cudaSuccess) return e;
-        int64_t want = (M.n_tasks + MV_THREADS - 1) / MV_THREADS;
-        int grid = per_sm * num_sms;
-        if (grid > want) grid = (int)want;
-        if (grid < 1) grid = 1;
-        kern<<<grid, MV_THREADS, smem, s>>>(M);
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        const int64_t want = (M.n_tasks + MV_THREADS - 1) / MV_THREADS;
+        const int64_t grid = (int64_t)per_sm * num_sms;
+        k_mv_eval<<<(int)(grid < want ? grid : want), MV_THREADS, smem, s>>>(M);
     }
     return cudaGetLastError();
 }

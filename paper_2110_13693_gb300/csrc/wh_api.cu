@@ -434,21 +434,17 @@ int prepare_moves(wh_layout* h, const wh_orders& o, const wh_plans& p, const int
 
 namespace {
 
-// The long tasks listed by the short-task pass: read their number (one
-// stream synchronisation), size the record matrix, run the record and DP
-// kernels, then the final status pass.
+// The long tasks listed by k_mv_eval: a record matrix for as many as are
+// ever common (tasks past it are scored by one lane each), the record and DP
+// kernels, which read the list's length on the device, then the final status
+// pass.
+constexpr int64_t kLongRecTasks = 1 << 16;
+
 int eval_long_tasks(wh_layout* h, wh::MoveArgs& M, cudaStream_t s) {
-    int32_t n_long = 0;
-    if (M.n_tasks > 0) {
-        if (cudaMemcpyAsync(&n_long, M.long_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return WH_ECUDA;
-        n_long = std::min(n_long, M.long_cap);
-    }
-    M.long_rec_cap = n_long;
-    if (n_long > 0) {
-        const size_t rec = align_up(sizeof(uint2) * (size_t)wh::MVL_RMAX * (size_t)n_long);
-        const size_t col = align_up(sizeof(int32_t) * (size_t)n_long);
+    M.long_rec_cap = (int32_t)std::min<int64_t>(M.n_tasks, kLongRecTasks);
+    if (M.long_rec_cap > 0) {
+        const size_t rec = align_up(sizeof(uint2) * (size_t)wh::MVL_RMAX * (size_t)M.long_rec_cap);
+        const size_t col = align_up(sizeof(int32_t) * (size_t)M.long_rec_cap);
         const int rc = grow(&h->mv_long, &h->mv_long_bytes, rec + 2 * col);
         if (rc != WH_OK) return rc;
         char* b = static_cast<char*>(h->mv_long);
@@ -480,8 +476,7 @@ extern "C" int wh_eval_moves(wh_layout* h, const wh_orders* orders, const wh_pla
     if (rc != WH_OK) return rc;
     M.tour_s_old = tour_s;
     M.tour_rr_old = tour_rr;
-    const bool k16 = wh::key16_ok(h->g);
-    if (wh::launch_moves_eval(M, k16, h->num_sms, s) != cudaSuccess) return WH_ECUDA;
+    if (wh::launch_moves_eval(M, h->num_sms, s) != cudaSuccess) return WH_ECUDA;
     rc = eval_long_tasks(h, M, s);
     if (rc != WH_OK) return rc;
     h->last_moves = moves;
@@ -648,7 +643,7 @@ extern "C" int wh_surrogate_screen_eval(wh_layout* h, wh_surrogate* sg, const wh
     if (rc != WH_OK) return rc;
     M.tour_s_old = tour_s;
     M.tour_rr_old = tour_rr;
-    if (wh::launch_moves_eval(M, wh::key16_ok(h->g), h->num_sms, s) != cudaSuccess) return WH_ECUDA;
+    if (wh::launch_moves_eval(M, h->num_sms, s) != cudaSuccess) return WH_ECUDA;
     rc = eval_long_tasks(h, M, s);
     if (rc != WH_OK) return rc;
     h->last_moves = kept;

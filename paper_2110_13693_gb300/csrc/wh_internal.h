@@ -128,7 +128,7 @@ struct MoveArgs {
     int4* tasks;                // [n_tasks]
     int2* task_cost;            // [n_tasks]: new (S-shape, optimal) cost of the task's tour, -1 if not counted
     int64_t n_tasks;
-    int32_t* long_list;         // tasks over SHORT_MAX lines
+    int32_t* long_list;         // tasks over ROW_MAXN lines
     int32_t* long_count;
     int32_t long_cap;
     // long tasks' per-aisle records for the one-task-per-thread DP: record r
@@ -248,8 +248,8 @@ cudaError_t launch_ls_apply(const LsArgs& L, cudaStream_t s);
 // checks, task counts and offsets; reuse_index: the index of the same plans
 // and order book is already in M's buffers, only the rest runs
 cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s, bool reuse_index);
-// task fill + tasks of <= SHORT_MAX lines; the long ones are listed
-cudaError_t launch_moves_eval(const MoveArgs& M, bool k16, int num_sms, cudaStream_t s);
+// task fill + tasks of <= ROW_MAXN lines; the long ones are listed
+cudaError_t launch_moves_eval(const MoveArgs& M, int num_sms, cudaStream_t s);
 // the listed long tasks (records, then their DPs) and the final status pass
 cudaError_t launch_moves_long(const MoveArgs& M, int num_sms, cudaStream_t s);
 constexpr int MVL_RMAX = 48;    // records per long task kept for the per-thread DP
