@@ -23,16 +23,6 @@ namespace wh {
 
 namespace {
 
-constexpr int MV_THREADS = 128;
-
-__device__ __forceinline__ int order_lines_checked(const EvalArgs& a, int o, int& lb, int& le) {
-    if ((unsigned)o >= (unsigned)a.n_orders) return -1;
-    lb = a.order_off[o];
-    le = a.order_off[o + 1];
-    if (lb < 0 || le < lb || le > a.n_lines) return -1;
-    return le - lb;
-}
-
 // plan of global tour t: largest p with plan_tour_off[p] <= t
 __device__ __forceinline__ int plan_of_tour(const EvalArgs& a, int t) {
     int lo = 0, hi = a.n_plans - 1;
@@ -137,61 +127,31 @@ __global__ void k_mv_sku_count(MoveArgs M) {
     }
 }
 
-// one block: exclusive scan of the per-SKU counts into sku_off, cursors
-// reset.  16 SKUs a thread and round, read and written 16 bytes at a time:
-// 50,000 SKUs in four rounds (one SKU a thread took 49 rounds, 49 us).
-constexpr int SKU_SCAN_T = 1024, SKU_SCAN_V = 16;
+// Places in sku_orders for every SKU's orders: a block scan of 1,024 SKUs'
+// counts and one atomic a block for its place among the blocks (the lists'
+// order does not matter), cursors reset.  One block scanning all of 50,000
+// SKUs in turn took 49 us, 21 us with 16 SKUs a thread.
+constexpr int SKU_ALLOC_T = 1024;
 
-__global__ void __launch_bounds__(SKU_SCAN_T) k_mv_sku_scan(MoveArgs M) {
+__global__ void __launch_bounds__(SKU_ALLOC_T) k_mv_sku_alloc(MoveArgs M) {
     __shared__ int warp_tot[32];
+    __shared__ int s_base;
     const int n = M.a.n_sku, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    int carry = 0;
-    for (int base = 0; base < n; base += SKU_SCAN_T * SKU_SCAN_V) {
-        const int i0 = base + tid * SKU_SCAN_V;
-        int v[SKU_SCAN_V], sum = 0;
-#pragma unroll
-        for (int u = 0; u < SKU_SCAN_V; u += 4) {
-            int4 x = make_int4(0, 0, 0, 0);
-            if (i0 + u + 4 <= n) x = *reinterpret_cast<const int4*>(M.sku_cur + i0 + u);
-            else {
-                if (i0 + u < n) x.x = M.sku_cur[i0 + u];
-                if (i0 + u + 1 < n) x.y = M.sku_cur[i0 + u + 1];
-                if (i0 + u + 2 < n) x.z = M.sku_cur[i0 + u + 2];
-            }
-            v[u] = x.x;
-            v[u + 1] = x.y;
-            v[u + 2] = x.z;
-            v[u + 3] = x.w;
-        }
-#pragma unroll
-        for (int u = 0; u < SKU_SCAN_V; ++u) sum += v[u];
-        const int incl = warp_inclusive_scan(sum);
-        if (lane == 31) warp_tot[w] = incl;
-        __syncthreads();
-        const int t = warp_tot[lane];
-        const int tot = warp_inclusive_scan(t);
-        int e = carry + incl - sum + __shfl_sync(0xffffffffu, tot - t, w);
-        carry += __shfl_sync(0xffffffffu, tot, 31);
-#pragma unroll
-        for (int u = 0; u < SKU_SCAN_V; u += 4) {
-            const int4 x = make_int4(e, e + v[u], e + v[u] + v[u + 1], e + v[u] + v[u + 1] + v[u + 2]);
-            e = x.w + v[u + 3];
-            if (i0 + u + 4 <= n) {
-                *reinterpret_cast<int4*>(M.sku_off + i0 + u) = x;
-                *reinterpret_cast<int4*>(M.sku_cur + i0 + u) = make_int4(0, 0, 0, 0);
-            } else {
-                const int xs[3] = {x.x, x.y, x.z};
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    if (i0 + u + k >= n) continue;
-                    M.sku_off[i0 + u + k] = xs[k];
-                    M.sku_cur[i0 + u + k] = 0;
-                }
-            }
-        }
-        __syncthreads();
+    const int i = blockIdx.x * SKU_ALLOC_T + tid;
+    const int v = i < n ? M.sku_cur[i] : 0;
+    const int incl = warp_inclusive_scan(v);
+    if (lane == 31) warp_tot[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        const int t = warp_tot[lane], tot = warp_inclusive_scan(t);
+        warp_tot[lane] = tot - t;
+        if (lane == 31) s_base = tot ? atomicAdd(&M.sku_cur[n], tot) : 0;
     }
-    if (tid == 0) M.sku_off[n] = carry;
+    __syncthreads();
+    if (i < n) {
+        M.sku_off[i] = s_base + warp_tot[w] + incl - v;
+        M.sku_cur[i] = 0;
+    }
 }
 
 __global__ void k_mv_sku_fill(MoveArgs M) {
@@ -202,8 +162,11 @@ __global__ void k_mv_sku_fill(MoveArgs M) {
         for (int l = lb; l < le; ++l) {
             const int s = a.line_sku[l];
             if ((unsigned)s >= (unsigned)a.n_sku) continue;
-            const int k = atomicAdd(&M.sku_cur[s], 1);
-            M.sku_orders[M.sku_off[s] + k] = o;
+            // (orders with malformed, overlapping line ranges hold more lines
+            // than there are)
+            const int k = M.sku_off[s] + atomicAdd(&M.sku_cur[s], 1);
+            if (k < a.n_lines) M.sku_orders[k] = o;
+            else atomicSub(&M.sku_cur[s], 1);
         }
     }
 }
@@ -250,7 +213,7 @@ __global__ void k_mv_count(MoveArgs M) {
                     if (mv.y == mv.z) st = 2;
                     else {
                         st = 0;
-                        cnt = (M.sku_off[mv.y + 1] - M.sku_off[mv.y]) + (M.sku_off[mv.z + 1] - M.sku_off[mv.z]);
+                        cnt = M.sku_cur[mv.y] + M.sku_cur[mv.z];
                     }
                 }
             } else if (mv.x == 3) {
@@ -262,7 +225,7 @@ __global__ void k_mv_count(MoveArgs M) {
                     if (a.slot_map[(int64_t)p * a.slot_stride + mv.y] == mv.z) st = 2;
                     else if (!used) {
                         st = 0;
-                        cnt = M.sku_off[mv.y + 1] - M.sku_off[mv.y];
+                        cnt = M.sku_cur[mv.y];
                     }
                 }
             }
@@ -342,20 +305,22 @@ __global__ void k_scan_add(int64_t* v, int64_t n, const int64_t* block_tot) {
 
 // task = {move, tour, order, tag}: tag >= 0 or -1: order moves (tag = order
 // removed, order = order added, -1 = none); tag -2 / -3: SKU swap, `order` is
-// the order of s1's / s2's list the task came from.  One move per lane; a SKU
-// list longer than MVF_SERIAL orders (a popular SKU can sit in hundreds) is
-// written by the whole warp, 32 tasks a step, at the same places.
-constexpr int MVF_SERIAL = 32;
+// the order of s1's / s2's list the task came from.  One move per lane, on
+// `unit` lanes of a warp (few where there are few moves); a SKU list longer
+// than MVF_SERIAL orders (a popular SKU can sit in hundreds) is written by the
+// whole warp, 32 tasks a step, at the same places.
+constexpr int MVF_SERIAL = 8;
 
-__global__ void k_mv_fill(MoveArgs M) {
+__global__ void k_mv_fill(MoveArgs M, int unit) {
     const EvalArgs& a = M.a;
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < M.n_moves; base += stride) {
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * unit; base < M.n_moves;
+         base += warps * unit) {
         const int m = (int)(base + lane);
         int lb[2] = {0, 0}, ln[2] = {0, 0}, lk[2] = {0, 0};   // a long list per side: begin, length, first task
         int64_t row = 0, t0 = 0;
-        if (m < M.n_moves && M.mstatus[m] == 0) {
+        if (lane < unit && m < M.n_moves && M.mstatus[m] == 0) {
             const int4 mv = M.moves[m];
             row = (int64_t)mv.w * a.n_orders;
             t0 = M.task_off[m];
@@ -372,7 +337,7 @@ __global__ void k_mv_fill(MoveArgs M) {
                 int k = 0;
                 for (int side = 0; side < (mv.x == 2 ? 2 : 1); ++side) {
                     const int sk = side ? mv.z : mv.y;
-                    const int b = M.sku_off[sk], e = M.sku_off[sk + 1];
+                    const int b = M.sku_off[sk], e = b + M.sku_cur[sk];
                     if (e - b > MVF_SERIAL) {
                         lb[side] = b;
                         ln[side] = e - b;
@@ -417,37 +382,34 @@ __device__ __forceinline__ int task_loc(const int32_t* map, int s, const int4 mv
 // the line's SKU is one the SKU move changes
 __device__ __forceinline__ bool sku_hit(int s, const int4 mv) { return s == mv.y || (mv.x == 2 && s == mv.z); }
 
-// Tasks of at most ROW_MAXN lines: a warp takes 32 tasks, one a lane, and
-// runs them together, as many of one plan at a time as its rows of shared
-// memory hold.  Task by task the lanes take the changed tour's orders (the
-// next task's ids in flight) and put its lines' SKUs, the moved ones already
-// exchanged, into the task's row; then the slot-map gathers of all rows run
-// flat, eight a lane in flight; then the rows are sorted (sort_rows) and each
-// lane costs its own task.  Few registers and no dependent gather per line:
-// 585,000 tasks of 262,144 moves at paper scale (60 lines each) took 505 us
-// one task a thread plus 180 us for the third of them with over 64 lines or
-// 32 aisles.
-constexpr int MV_WARPS = MV_THREADS / 32;
-constexpr int MV_ROWS = 2048;              // keys of a warp's rows: 32 tours of 64 lines
-constexpr uint32_t SKU_BAD = 0x7FFFFFFFu;  // in a row before the gathers: unusable SKU
-constexpr uint32_t SKU_AT = 0x80000000u;   // a relocated SKU: SKU_AT | its location
+// The changed tour of a lane's task: its sequence range, the order added and a
+// bound on its lines; ok is cleared when its orders are malformed.
+__device__ __forceinline__ void task_tour(const MoveArgs& M, bool has, RowTour& w, bool& ok) {
+    const EvalArgs& a = M.a;
+    w.q0 = w.q1 = w.ub = 0;
+    w.add = has && w.mv.x < 2 && w.tk.z >= 0 ? w.tk.z : -1;
+    if (!has) return;
+    w.q0 = a.tour_off[w.tk.y];
+    w.q1 = a.tour_off[w.tk.y + 1];
+    int lb, le;
+    const int cur = M.tour_lines[w.tk.y], more = w.add >= 0 ? order_lines_checked(a, w.add, lb, le) : 0;
+    ok = cur >= 0 && more >= 0;
+    w.ub = ok ? cur + more : 0;
+}
 
-__global__ void __launch_bounds__(MV_THREADS, 5) k_mv_eval(MoveArgs M) {
+// Tasks of at most ROW_MAXN lines: up to 32 a warp, one a lane, read, sorted
+// (run_rows) and costed together.
+__global__ void __launch_bounds__(ROW_THREADS, 5) k_mv_eval(MoveArgs M, int unit) {
     extern __shared__ __align__(16) uint32_t mv_rows[];
-    __shared__ uint16_t s_base[MV_WARPS][32], s_list[MV_WARPS][32];
-    __shared__ uint8_t s_n[MV_WARPS][32];
+    __shared__ RowList s_rl[ROW_WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    uint32_t* rows = mv_rows + wid * MV_ROWS;
-    uint16_t* bases = s_base[wid];
-    uint16_t* list = s_list[wid];
-    uint8_t* ns = s_n[wid];
+    uint32_t* rows = mv_rows + wid * ROW_WORDS;
     const EvalArgs& a = M.a;
     const DPConst c = dp_const(a.g);
-    const int64_t stride = (int64_t)gridDim.x * MV_WARPS * 32;
-    for (int64_t u0 = ((int64_t)blockIdx.x * MV_WARPS + wid) * 32; u0 < M.n_tasks; u0 += stride) {
+    const int64_t stride = (int64_t)gridDim.x * ROW_WARPS * unit;
+    for (int64_t u0 = ((int64_t)blockIdx.x * ROW_WARPS + wid) * unit; u0 < M.n_tasks; u0 += stride) {
         const int64_t i = u0 + lane;
-        const bool active = i < M.n_tasks;
+        const bool active = lane < unit && i < M.n_tasks;
         int4 tk = make_int4(-1, -1, -1, -1), mv = make_int4(0, 0, 0, 0);
         if (active) {
             tk = M.tasks[i];
@@ -455,20 +417,12 @@ __global__ void __launch_bounds__(MV_THREADS, 5) k_mv_eval(MoveArgs M) {
         }
         // an order of the SKU lists outside the plan: nothing to cost
         const bool has = active && tk.y >= 0 && tk.y < a.n_tours;
-        const bool sku_move = mv.x >= 2;
         bool ok = active;
-        int q0 = 0, q1 = 0, ub = 0;   // ub: the changed tour has at most this many lines
-        const int add = has && !sku_move && tk.z >= 0 ? tk.z : -1;
-        if (has) {
-            q0 = a.tour_off[tk.y];
-            q1 = a.tour_off[tk.y + 1];
-            ub = M.tour_lines[tk.y];
-            int lb, le;
-            const int ca = add >= 0 ? order_lines_checked(a, add, lb, le) : 0;
-            ok = ub >= 0 && ca >= 0;
-            ub = ok ? ub + ca : 0;
-        }
-        const bool lng = has && ok && ub > ROW_MAXN;
+        RowTour w;
+        w.tk = tk;
+        w.mv = mv;
+        task_tour(M, has, w, ok);
+        const bool lng = has && ok && w.ub > ROW_MAXN;
         if (lng) {
             const int slot = atomicAdd(M.long_count, 1);
             if (slot < M.long_cap) M.long_list[slot] = (int32_t)i;
@@ -476,194 +430,16 @@ __global__ void __launch_bounds__(MV_THREADS, 5) k_mv_eval(MoveArgs M) {
         }
         bool run = false;   // the task's cost counts: cs, cr
         int n = 0, cs = 0, cr = 0;
-        unsigned todo = __ballot_sync(0xffffffffu, has && ok && !lng);
-        while (todo) {
-            // the next tasks of one plan that fit the rows
-            const int plan = __shfl_sync(0xffffffffu, mv.w, __ffs(todo) - 1);
-            const bool cand = ((todo >> lane) & 1u) && mv.w == plan;
-            const int incl = warp_inclusive_scan(cand ? ub : 0);
-            const bool mine = cand && incl <= MV_ROWS;
-            const unsigned take = __ballot_sync(0xffffffffu, mine);
-            const int total = __shfl_sync(0xffffffffu, incl, 31 - __clz(take));
-            todo &= ~take;
-            const int base = mine ? incl - ub : 0;
-            const int32_t* map = a.slot_map + (int64_t)plan * a.slot_stride;
-            bool primary = true;
-            // ids two tasks ahead, line ranges one task ahead
-            int j = __ffs(take) - 1, j2 = j;
-            unsigned left = take & (take - 1);
-            auto first_ids = [&](int k) {
-                const int b0 = __shfl_sync(0xffffffffu, q0, k), b1 = __shfl_sync(0xffffffffu, q1, k);
-                return b0 + lane < b1 ? a.order_seq[b0 + lane] : -1;
-            };
-            int o_cur = first_ids(j), o_nxt = -1;
-            int lb_cur = 0, le_cur = 0;
-            if (o_cur >= 0) {
-                lb_cur = a.order_off[o_cur];
-                le_cur = a.order_off[o_cur + 1];
-            }
-            if (left) {
-                j2 = __ffs(left) - 1;
-                o_nxt = first_ids(j2);
-            }
-            for (;;) {
-                const int b0 = __shfl_sync(0xffffffffu, q0, j), b1 = __shfl_sync(0xffffffffu, q1, j);
-                const int jadd = __shfl_sync(0xffffffffu, add, j), jbase = __shfl_sync(0xffffffffu, base, j);
-                const int type = __shfl_sync(0xffffffffu, mv.x, j);
-                const int mb = __shfl_sync(0xffffffffu, mv.y, j), mc = __shfl_sync(0xffffffffu, mv.z, j);
-                const int tz = __shfl_sync(0xffffffffu, tk.z, j), tw = __shfl_sync(0xffffffffu, tk.w, j);
-                const int jj = j;
-                const bool more = left != 0;
-                int o0 = o_cur, lb0 = lb_cur, le0 = le_cur;   // this lane's order of the first 32
-                j = j2;
-                o_cur = o_nxt;
-                lb_cur = le_cur = 0;
-                if (more) {
-                    if (o_cur >= 0) {
-                        lb_cur = a.order_off[o_cur];
-                        le_cur = a.order_off[o_cur + 1];
-                    }
-                    left &= left - 1;
-                    if (left) {
-                        j2 = __ffs(left) - 1;
-                        o_nxt = first_ids(j2);
-                    }
-                }
-                const bool swap = type >= 2;
-                const int rem = !swap && tw >= 0 ? tw : -1;
-                const int b_end = jadd >= 0 ? b1 + 1 : b1;
-                if (b0 + lane < b1) {
-                    if (o0 == rem) lb0 = le0 = 0;
-                } else if (b0 + lane < b_end) {   // the added order comes last
-                    o0 = jadd;
-                    lb0 = a.order_off[o0];
-                    le0 = a.order_off[o0 + 1];
-                }
-                uint32_t* row = rows + jbase;
-                // the lines' indices at their places (lanes over orders;
-                // ids and line counts were checked with the tour's count)
-                int cnt_all = 0;
-                for (int qb = b0; qb < b_end; qb += 32) {
-                    int lb = lb0, le = le0;
-                    if (qb > b0) {
-                        const int q = qb + lane;
-                        lb = le = 0;
-                        if (q < b_end) {
-                            const int o = q < b1 ? a.order_seq[q] : jadd;
-                            if (!(q < b1 && o == rem)) {
-                                lb = a.order_off[o];
-                                le = a.order_off[o + 1];
-                            }
-                        }
-                    }
-                    const int cnt = le - lb;
-                    const int inc = warp_inclusive_scan(cnt);
-                    uint32_t* w = row + cnt_all + inc - cnt;
-                    for (int l = lb; l < le; ++l) *w++ = (uint32_t)l;
-                    cnt_all += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                __syncwarp();
-                // their SKUs, the move applied: an exchanged SKU takes the
-                // other's place, a relocated one its new location
-                int hit_min = 0x7fffffff;
-                bool own_has_s1 = false;
-                for (int x0 = 0; x0 < cnt_all; x0 += 64) {
-                    int l[2];
-                    uint32_t sk[2];
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int x = x0 + 32 * u + lane;
-                        l[u] = x < cnt_all ? (int)row[x] : -1;
-                        sk[u] = l[u] >= 0 ? (uint32_t)a.line_sku[l[u]] : SKU_BAD;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        uint32_t k = sk[u] < (uint32_t)a.n_sku ? sk[u] : SKU_BAD;
-                        if (swap) {
-                            const bool s1 = k == (uint32_t)mb, hit = s1 || (type == 2 && k == (uint32_t)mc);
-                            // a moved SKU's line: the order that holds it
-                            // (a SKU move keeps every order of the tour)
-                            for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1) {
-                                const int src = __ffs(hits) - 1;
-                                const int hl = __shfl_sync(0xffffffffu, l[u], src);
-                                const bool h1 = __shfl_sync(0xffffffffu, (int)s1, src) != 0;
-                                for (int qb = b0; qb < b1; qb += 32) {
-                                    int o = o0, lb = lb0, le = le0;
-                                    if (qb > b0) {
-                                        lb = le = 0;
-                                        if (qb + lane < b1) {
-                                            o = a.order_seq[qb + lane];
-                                            lb = a.order_off[o];
-                                            le = a.order_off[o + 1];
-                                        }
-                                    }
-                                    if (hl >= lb && hl < le) {
-                                        hit_min = min(hit_min, o);
-                                        own_has_s1 |= h1 && o == tz;
-                                    }
-                                }
-                            }
-                            if (hit) k = type == 3 ? SKU_AT | (uint32_t)mc : (uint32_t)(s1 ? mc : mb);
-                        }
-                        if (l[u] >= 0) row[x0 + 32 * u + lane] = k;
-                    }
-                }
-                if (swap) {
-                    hit_min = __reduce_min_sync(0xffffffffu, hit_min);
-                    own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
-                }
-                if (lane == jj) {
-                    n = cnt_all;
-                    primary = !swap || (hit_min == tz && (tw == -2 || !own_has_s1));
-                }
-                if (!more) break;
-            }
-            __syncwarp();
-            // keys, all rows at once (what lies between rows is translated
-            // too and read by nobody)
-            bool bad = false;
-            for (int x0 = lane; x0 < total; x0 += 256) {
-                uint32_t sk[8];
-                int loc[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) sk[u] = x0 + 32 * u < total ? rows[x0 + 32 * u] : SKU_BAD;
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    loc[u] = sk[u] < (uint32_t)a.n_sku ? map[sk[u]] : ((sk[u] & SKU_AT) ? (int)(sk[u] & ~SKU_AT) : -1);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (x0 + 32 * u >= total) continue;
-                    const bool in = (uint32_t)loc[u] < (uint32_t)a.g.n_loc;
-                    bad |= !in;
-                    rows[x0 + 32 * u] = in ? loc_key(a.g, loc[u]) : KEY_BAD;
-                }
-            }
-            bad = __any_sync(0xffffffffu, bad);
-            // sort: the tasks that count, those over 64 lines first
-            const bool cost = mine && primary;
-            const unsigned big = __ballot_sync(0xffffffffu, cost && n > 64), all = __ballot_sync(0xffffffffu, cost);
-            const int n_big = __popc(big), n_all = __popc(all);
-            if (mine) {
-                bases[lane] = (uint16_t)base;
-                ns[lane] = (uint8_t)n;
-            }
-            if (cost) list[n > 64 ? __popc(big & lt_mask) : n_big + __popc(all & ~big & lt_mask)] = (uint16_t)lane;
-            __syncwarp();
-            for (int k = 0; k < n_all;) {
-                const int G = k < n_big ? 8 : 4, end = k < n_big ? n_big : n_all;
-                sort_rows(G, rows, list, bases, ns, k, end, lane);
-                k = min(k + 32 / G, end);
-            }
-            __syncwarp();
-            if (mine) {
-                const uint32_t* row = rows + base;
-                if (cost) row_costs(a.g, c, row, n, true, cs, cr);
-                if (bad)
-                    for (int p = 0; p < n; ++p) ok &= row[p] < KEY_BAD_SKU;
-                run = cost && ok;
-            }
-            __syncwarp();
-        }
+        run_rows(a, rows, s_rl[wid], w, __ballot_sync(0xffffffffu, has && ok && !lng), lane,
+                 [&](bool mine, bool primary, int base, int rn, bool bad) {
+                     if (!mine) return;
+                     const uint32_t* row = rows + base;
+                     n = rn;
+                     if (primary) row_costs(a.g, c, row, n, true, cs, cr);
+                     if (bad)
+                         for (int p = 0; p < n; ++p) ok &= row[p] < KEY_BAD_SKU;
+                     run = primary && ok;
+                 });
         if (active && !ok) {
             flag(a.status, WH_STATUS_BAD_ORDER);
             M.mstatus[tk.x] = 3;
@@ -952,7 +728,7 @@ cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s,
         k_mv_tours<<<grid_of(a.n_tours, 256), 256, 0, s>>>(M);
     }
     if (a.n_lines > 0) k_mv_sku_count<<<grid_of(a.n_lines, 256), 256, 0, s>>>(M);
-    k_mv_sku_scan<<<1, SKU_SCAN_T, 0, s>>>(M);
+    if (a.n_sku > 0) k_mv_sku_alloc<<<(a.n_sku + SKU_ALLOC_T - 1) / SKU_ALLOC_T, SKU_ALLOC_T, 0, s>>>(M);
     if (a.n_orders > 0) k_mv_sku_fill<<<grid_of(a.n_orders, 256), 256, 0, s>>>(M);
     k_mv_count<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
     // exclusive scan of n_moves + 1 task counts
@@ -964,24 +740,27 @@ cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s,
     return cudaGetLastError();
 }
 
-cudaError_t launch_moves_fill(const MoveArgs& M, cudaStream_t s) {
-    if (M.n_moves > 0) k_mv_fill<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
+// 32 warps an SM: enough to hide the lists' gathers, and up to 32 moves a
+// warp beyond that (16,384 kept moves 51 us with 32 moves a warp throughout)
+cudaError_t launch_moves_fill(const MoveArgs& M, int num_sms, cudaStream_t s) {
+    if (M.n_moves <= 0) return cudaSuccess;
+    const int64_t warps = (int64_t)num_sms * 32, u = (M.n_moves + warps - 1) / warps;
+    const int unit = u > 32 ? 32 : (int)u;
+    k_mv_fill<<<grid_of((M.n_moves + unit - 1) / unit * 32, 256), 256, 0, s>>>(M, unit);
     return cudaGetLastError();
 }
 
 cudaError_t launch_moves_eval(const MoveArgs& M, int num_sms, cudaStream_t s) {
-    if (M.n_moves > 0) k_mv_fill<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
+    const cudaError_t f = launch_moves_fill(M, num_sms, s);
+    if (f != cudaSuccess) return f;
     if (M.n_tasks > 0) {
-        const size_t smem = sizeof(uint32_t) * MV_ROWS * MV_WARPS;
-        cudaError_t e = cudaFuncSetAttribute(k_mv_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_eval, MV_THREADS, smem);
+        cudaError_t e = rows_per_sm(k_mv_eval, &per_sm);
         if (e != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        const int64_t want = (M.n_tasks + MV_THREADS - 1) / MV_THREADS;
         const int64_t grid = (int64_t)per_sm * num_sms;
-        k_mv_eval<<<(int)(grid < want ? grid : want), MV_THREADS, smem, s>>>(M);
+        const int unit = row_unit(M.n_tasks, grid * ROW_WARPS);
+        const int64_t want = (M.n_tasks + (int64_t)unit * ROW_WARPS - 1) / (unit * ROW_WARPS);
+        k_mv_eval<<<(int)(grid < want ? grid : want), ROW_THREADS, ROW_SMEM, s>>>(M, unit);
     }
     return cudaGetLastError();
 }
@@ -1226,11 +1005,13 @@ __global__ void __launch_bounds__(TF_THREADS) k_task_features(MoveArgs M, FeatCo
 // Predicted delta of every move (sum over its counted tasks, in order), then
 // per plan the `keep` moves with the lowest predicted delta (ties: lowest
 // index); unfilled places get an invalid move that scores status 3.
+constexpr int SCORE_SERIAL = 32;
+
 __global__ void k_screen_score(ScreenArgs S) {
     const MoveArgs& M = S.M;
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // one move per lane; a move of more than MVF_SERIAL tasks is scored by the
+    // one move per lane; a move of more than SCORE_SERIAL tasks is scored by the
     // whole warp: lanes load 32 tasks' terms at once, and every lane adds
     // them up in task order, so the sum is the serial one
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < M.n_moves; base += stride) {
@@ -1242,15 +1023,24 @@ __global__ void k_screen_score(ScreenArgs S) {
             i0 = M.task_off[m];
             i1 = M.task_off[m + 1];
         }
-        const bool lng = i1 - i0 > MVF_SERIAL;
+        const bool lng = i1 - i0 > SCORE_SERIAL;
         if (!lng)
-            for (int64_t i = i0; i < i1; ++i) {
-                const int4 tk = M.tasks[i];
-                if (tk.y < 0) continue;
-                // counted task: an order move, or the first task of its tour for a SKU swap
-                const int2 c = M.task_cost[i];
-                if (c.x < 0) continue;
-                sc += S.y_task[i] - S.y_tour[tk.y];
+            for (int64_t i = i0; i < i1; i += 4) {
+                // counted task: an order move, or the first task of its tour
+                // for a SKU swap; four tasks' loads in flight
+                int t[4];
+                float yt[4], yo[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    t[u] = i + u < i1 ? M.tasks[i + u].y : -1;
+                    if (i + u < i1 && M.task_cost[i + u].x < 0) t[u] = -1;
+                    yt[u] = i + u < i1 ? S.y_task[i + u] : 0.0f;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) yo[u] = t[u] >= 0 ? S.y_tour[t[u]] : 0.0f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (t[u] >= 0) sc += yt[u] - yo[u];
             }
         unsigned longs = __ballot_sync(0xffffffffu, lng);
         while (longs) {
@@ -1258,21 +1048,28 @@ __global__ void k_screen_score(ScreenArgs S) {
             longs &= longs - 1;
             const int64_t b = __shfl_sync(0xffffffffu, i0, src), e = __shfl_sync(0xffffffffu, i1, src);
             float acc = 0.0f;
-            for (int64_t c0 = b; c0 < e; c0 += 32) {
-                const int64_t i = c0 + lane;
-                float term = 0.0f;
-                bool counted = false;
-                if (i < e) {
-                    const int4 tk = M.tasks[i];
-                    if (tk.y >= 0 && M.task_cost[i].x >= 0) {
-                        counted = true;
-                        term = S.y_task[i] - S.y_tour[tk.y];
-                    }
+            for (int64_t c0 = b; c0 < e; c0 += 128) {
+                // 128 tasks' terms in flight (a popular SKU's move has
+                // hundreds of tasks, and the longest sets the kernel's time)
+                int t[4];
+                float term[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t i = c0 + 32 * u + lane;
+                    t[u] = i < e && M.task_cost[i].x >= 0 ? M.tasks[i].y : -1;
+                    term[u] = i < e ? S.y_task[i] : 0.0f;
                 }
-                const unsigned cm = __ballot_sync(0xffffffffu, counted);
-                for (int j = 0; j < 32; ++j) {
-                    const float tj = __shfl_sync(0xffffffffu, term, j);
-                    if ((cm >> j) & 1u) acc += tj;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (t[u] >= 0) term[u] -= S.y_tour[t[u]];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned cm = __ballot_sync(0xffffffffu, t[u] >= 0);
+#pragma unroll 8
+                    for (int j = 0; j < 32; ++j) {
+                        const float tj = __shfl_sync(0xffffffffu, term[u], j);
+                        if ((cm >> j) & 1u) acc += tj;
+                    }
                 }
             }
             if (lane == src) sc = acc;

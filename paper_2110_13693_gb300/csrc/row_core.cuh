@@ -101,5 +101,255 @@ __device__ __forceinline__ void row_costs(const Geo& g, const DPConst& c, const 
     cr = need_rr ? dp_final(v) + c.p2 * pa : 0;
 }
 
+// ------------------------------------------------- a warp's rows of tours
+// A warp takes up to 32 tours, one a lane, possibly changed by a move, as
+// many of one plan at a time as its rows of shared memory hold.  Tour by tour
+// the lanes take the tour's orders (the next tours' ids and line ranges in
+// flight) and put its lines' SKUs, the moved ones already exchanged, into the
+// tour's row; then the slot-map gathers of all rows run flat, eight a lane in
+// flight; then the rows are sorted (sort_rows).  No dependent gather per line
+// and few registers.
+constexpr int ROW_WARPS = 4;                // warps of a CTA
+constexpr int ROW_THREADS = ROW_WARPS * 32;
+constexpr int ROW_WORDS = 2048;             // keys of a warp's rows: 32 tours of 64 lines
+constexpr uint32_t SKU_BAD = 0x7FFFFFFFu;   // in a row before the gathers: unusable SKU
+constexpr uint32_t SKU_AT = 0x80000000u;    // a relocated SKU: SKU_AT | its location
+constexpr size_t ROW_SMEM = sizeof(uint32_t) * ROW_WORDS * ROW_WARPS;
+
+// per warp, in shared memory
+struct RowList {
+    uint16_t base[32], list[32];
+    uint8_t n[32];
+};
+
+// A lane's tour: sequence positions q0 .. q1 - 1 of checked order ids, at most
+// ub <= ROW_MAXN lines.  mv: {type, a, b, plan} of the move that changes it
+// (type 0 for none), tk: {-, -, order of the move's list or -, order removed
+// or list tag or -1}; add: the order added, or -1.
+struct RowTour {
+    int q0, q1, ub, add;
+    int4 tk, mv;
+};
+
+__device__ __forceinline__ int order_lines_checked(const EvalArgs& a, int o, int& lb, int& le) {
+    if ((unsigned)o >= (unsigned)a.n_orders) return -1;
+    lb = a.order_off[o];
+    le = a.order_off[o + 1];
+    if (lb < 0 || le < lb || le > a.n_lines) return -1;
+    return le - lb;
+}
+
+// Tours per warp and turn that give every warp of the grid work (32 where
+// there is enough: a warp reads its tours one after another).
+inline int row_unit(int64_t items, int64_t warps) {
+    const int64_t u = (items + warps - 1) / warps;
+    return u < 4 ? 4 : u > 32 ? 32 : (int)u;
+}
+
+// CTAs per SM of a kernel over rows
+template <typename K>
+cudaError_t rows_per_sm(K kern, int* per_sm) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ROW_SMEM);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, ROW_THREADS, ROW_SMEM);
+    if (e == cudaSuccess && *per_sm < 1) e = cudaErrorInvalidConfiguration;
+    return e;
+}
+
+// Runs the lanes of `todo`.  For every batch done(mine, primary, base, n, bad)
+// is called by the whole warp: whether this lane's task is in the batch,
+// whether it is the counted one of its tour (only those rows are sorted), its
+// row's place and length, and whether some row holds a line without a usable
+// location (it sorts to its row's end).
+template <typename Done>
+__device__ __forceinline__ void run_rows(const EvalArgs& a, uint32_t* rows, RowList& rl, const RowTour& w, unsigned todo,
+                                         int lane, Done done) {
+    const unsigned lt_mask = (1u << lane) - 1u;
+    uint16_t* bases = rl.base;
+    uint16_t* list = rl.list;
+    uint8_t* ns = rl.n;
+    while (todo) {
+        // the next tasks of one plan that fit the rows
+        const int plan = __shfl_sync(0xffffffffu, w.mv.w, __ffs(todo) - 1);
+        const bool cand = ((todo >> lane) & 1u) && w.mv.w == plan;
+        const int incl = warp_inclusive_scan(cand ? w.ub : 0);
+        const bool mine = cand && incl <= ROW_WORDS;
+        const unsigned take = __ballot_sync(0xffffffffu, mine);
+        const int total = __shfl_sync(0xffffffffu, incl, 31 - __clz(take));
+        todo &= ~take;
+        const int base = mine ? incl - w.ub : 0;
+        const int32_t* map = a.slot_map + (int64_t)plan * a.slot_stride;
+        bool primary = true;
+        int n = 0;
+        // ids two tasks ahead, line ranges one task ahead
+        int j = __ffs(take) - 1, j2 = j;
+        unsigned left = take & (take - 1);
+        auto first_ids = [&](int k) {
+            const int b0 = __shfl_sync(0xffffffffu, w.q0, k), b1 = __shfl_sync(0xffffffffu, w.q1, k);
+            return b0 + lane < b1 ? a.order_seq[b0 + lane] : -1;
+        };
+        int o_cur = first_ids(j), o_nxt = -1;
+        int lb_cur = 0, le_cur = 0;
+        if (o_cur >= 0) {
+            lb_cur = a.order_off[o_cur];
+            le_cur = a.order_off[o_cur + 1];
+        }
+        if (left) {
+            j2 = __ffs(left) - 1;
+            o_nxt = first_ids(j2);
+        }
+        for (;;) {
+            const int b0 = __shfl_sync(0xffffffffu, w.q0, j), b1 = __shfl_sync(0xffffffffu, w.q1, j);
+            const int jadd = __shfl_sync(0xffffffffu, w.add, j), jbase = __shfl_sync(0xffffffffu, base, j);
+            const int type = __shfl_sync(0xffffffffu, w.mv.x, j);
+            const int mb = __shfl_sync(0xffffffffu, w.mv.y, j), mc = __shfl_sync(0xffffffffu, w.mv.z, j);
+            const int tz = __shfl_sync(0xffffffffu, w.tk.z, j), tw = __shfl_sync(0xffffffffu, w.tk.w, j);
+            const int jj = j;
+            const bool more = left != 0;
+            int o0 = o_cur, lb0 = lb_cur, le0 = le_cur;   // this lane's order of the first 32
+            j = j2;
+            o_cur = o_nxt;
+            lb_cur = le_cur = 0;
+            if (more) {
+                if (o_cur >= 0) {
+                    lb_cur = a.order_off[o_cur];
+                    le_cur = a.order_off[o_cur + 1];
+                }
+                left &= left - 1;
+                if (left) {
+                    j2 = __ffs(left) - 1;
+                    o_nxt = first_ids(j2);
+                }
+            }
+            const bool swap = type >= 2;
+            const int rem = !swap && tw >= 0 ? tw : -1;
+            const int b_end = jadd >= 0 ? b1 + 1 : b1;
+            if (b0 + lane < b1) {
+                if (o0 == rem) lb0 = le0 = 0;
+            } else if (b0 + lane < b_end) {   // the added order comes last
+                o0 = jadd;
+                lb0 = a.order_off[o0];
+                le0 = a.order_off[o0 + 1];
+            }
+            uint32_t* row = rows + jbase;
+            // the lines' indices at their places (lanes over orders;
+            // ids and line counts were checked with the tour's count)
+            int cnt_all = 0;
+            for (int qb = b0; qb < b_end; qb += 32) {
+                int lb = lb0, le = le0;
+                if (qb > b0) {
+                    const int q = qb + lane;
+                    lb = le = 0;
+                    if (q < b_end) {
+                        const int o = q < b1 ? a.order_seq[q] : jadd;
+                        if (!(q < b1 && o == rem)) {
+                            lb = a.order_off[o];
+                            le = a.order_off[o + 1];
+                        }
+                    }
+                }
+                const int cnt = le - lb;
+                const int inc = warp_inclusive_scan(cnt);
+                uint32_t* at = row + cnt_all + inc - cnt;
+                for (int l = lb; l < le; ++l) *at++ = (uint32_t)l;
+                cnt_all += __shfl_sync(0xffffffffu, inc, 31);
+            }
+            __syncwarp();
+            // their SKUs, the move applied: an exchanged SKU takes the
+            // other's place, a relocated one its new location
+            int hit_min = 0x7fffffff;
+            bool own_has_s1 = false;
+            for (int x0 = 0; x0 < cnt_all; x0 += 64) {
+                int l[2];
+                uint32_t sk[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int x = x0 + 32 * u + lane;
+                    l[u] = x < cnt_all ? (int)row[x] : -1;
+                    sk[u] = l[u] >= 0 ? (uint32_t)a.line_sku[l[u]] : SKU_BAD;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    uint32_t k = sk[u] < (uint32_t)a.n_sku ? sk[u] : SKU_BAD;
+                    if (swap) {
+                        const bool s1 = k == (uint32_t)mb, hit = s1 || (type == 2 && k == (uint32_t)mc);
+                        // a moved SKU's line: the order that holds it
+                        // (a SKU move keeps every order of the tour)
+                        for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1) {
+                            const int src = __ffs(hits) - 1;
+                            const int hl = __shfl_sync(0xffffffffu, l[u], src);
+                            const bool h1 = __shfl_sync(0xffffffffu, (int)s1, src) != 0;
+                            for (int qb = b0; qb < b1; qb += 32) {
+                                int o = o0, lb = lb0, le = le0;
+                                if (qb > b0) {
+                                    lb = le = 0;
+                                    if (qb + lane < b1) {
+                                        o = a.order_seq[qb + lane];
+                                        lb = a.order_off[o];
+                                        le = a.order_off[o + 1];
+                                    }
+                                }
+                                if (hl >= lb && hl < le) {
+                                    hit_min = min(hit_min, o);
+                                    own_has_s1 |= h1 && o == tz;
+                                }
+                            }
+                        }
+                        if (hit) k = type == 3 ? SKU_AT | (uint32_t)mc : (uint32_t)(s1 ? mc : mb);
+                    }
+                    if (l[u] >= 0) row[x0 + 32 * u + lane] = k;
+                }
+            }
+            if (swap) {
+                hit_min = __reduce_min_sync(0xffffffffu, hit_min);
+                own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
+            }
+            if (lane == jj) {
+                n = cnt_all;
+                primary = !swap || (hit_min == tz && (tw == -2 || !own_has_s1));
+            }
+            if (!more) break;
+        }
+        __syncwarp();
+        // keys, all rows at once (what lies between rows is translated
+        // too and read by nobody)
+        bool bad = false;
+        for (int x0 = lane; x0 < total; x0 += 256) {
+            uint32_t sk[8];
+            int loc[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sk[u] = x0 + 32 * u < total ? rows[x0 + 32 * u] : SKU_BAD;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                loc[u] = sk[u] < (uint32_t)a.n_sku ? map[sk[u]] : ((sk[u] & SKU_AT) ? (int)(sk[u] & ~SKU_AT) : -1);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (x0 + 32 * u >= total) continue;
+                const bool in = (uint32_t)loc[u] < (uint32_t)a.g.n_loc;
+                bad |= !in;
+                rows[x0 + 32 * u] = in ? loc_key(a.g, loc[u]) : KEY_BAD;
+            }
+        }
+        bad = __any_sync(0xffffffffu, bad);
+        // sort: those over 64 lines first
+        const bool cost = mine && primary;
+        const unsigned big = __ballot_sync(0xffffffffu, cost && n > 64), all = __ballot_sync(0xffffffffu, cost);
+        const int n_big = __popc(big), n_all = __popc(all);
+        if (mine) {
+            bases[lane] = (uint16_t)base;
+            ns[lane] = (uint8_t)n;
+        }
+        if (cost) list[n > 64 ? __popc(big & lt_mask) : n_big + __popc(all & ~big & lt_mask)] = (uint16_t)lane;
+        __syncwarp();
+        for (int k = 0; k < n_all;) {
+            const int G = k < n_big ? 8 : 4, end = k < n_big ? n_big : n_all;
+            sort_rows(G, rows, list, bases, ns, k, end, lane);
+            k = min(k + 32 / G, end);
+        }
+        __syncwarp();
+        done(mine, primary, base, n, bad);
+        __syncwarp();
+    }
+}
+
 }  // namespace
 }  // namespace wh

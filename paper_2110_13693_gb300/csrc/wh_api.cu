@@ -513,7 +513,7 @@ int screen_moves(wh_layout* h, wh_surrogate* sg, const wh_orders& o, const wh_pl
         rc = prepare_moves(h, o, p, moves, n_moves, max_orders, max_lines, dl, st, M, s);
         if (rc != WH_OK) return rc;
     }
-    if (wh::launch_moves_fill(M, s) != cudaSuccess) return WH_ECUDA;
+    if (wh::launch_moves_fill(M, h->num_sms, s) != cudaSuccess) return WH_ECUDA;
     // features and predictions of the current tours and of the tasks' changed tours
     const size_t need = head + align_up(feat_row * (size_t)(p.n_tours + 1)) + align_up(sizeof(float) * (size_t)(p.n_tours + 1)) +
                         align_up(feat_row * (size_t)(M.n_tasks + 1)) + align_up(sizeof(float) * (size_t)(M.n_tasks + 1)) +
@@ -528,7 +528,7 @@ int screen_moves(wh_layout* h, wh_surrogate* sg, const wh_orders& o, const wh_pl
         int64_t* dl = reinterpret_cast<int64_t*>(b + align_up(sizeof(int32_t) * (size_t)n_moves));
         rc = prepare_moves(h, o, p, moves, n_moves, max_orders, max_lines, dl, st, M, s);
         if (rc != WH_OK) return rc;
-        if (wh::launch_moves_fill(M, s) != cudaSuccess) return WH_ECUDA;
+        if (wh::launch_moves_fill(M, h->num_sms, s) != cudaSuccess) return WH_ECUDA;
     }
     char* b = static_cast<char*>(h->sr_scratch);
     size_t at = align_up(sizeof(int32_t) * (size_t)n_moves) + align_up(sizeof(int64_t) * 2 * (size_t)n_moves);

@@ -120,8 +120,8 @@ struct MoveArgs {
     // scratch
     int32_t* order_tour;        // [n_plans][n_orders]: global tour holding the order, -1 if none
     int32_t* tour_lines;        // [n_tours]: lines of the tour, -1 if malformed
-    int32_t* sku_off;           // [n_sku+1]: SKU -> orders index
-    int32_t* sku_cur;           // [n_sku+1]: counts, then fill cursors
+    int32_t* sku_off;           // [n_sku]: first of a SKU's orders in sku_orders
+    int32_t* sku_cur;           // [n_sku+1]: counts, then fill cursors, at last the lists' lengths; [n_sku]: places given
     int32_t* sku_orders;        // [n_lines]
     int64_t* task_off;          // [n_moves+1]: exclusive scan of task counts
     int64_t* scan_aux;          // block totals of that scan
@@ -253,7 +253,7 @@ cudaError_t launch_moves_eval(const MoveArgs& M, int num_sms, cudaStream_t s);
 // the listed long tasks (records, then their DPs) and the final status pass
 cudaError_t launch_moves_long(const MoveArgs& M, int num_sms, cudaStream_t s);
 constexpr int MVL_RMAX = 48;    // records per long task kept for the per-thread DP
-cudaError_t launch_moves_fill(const MoveArgs& M, cudaStream_t s);
+cudaError_t launch_moves_fill(const MoveArgs& M, int num_sms, cudaStream_t s);
 
 // Surrogate (k_surrogate.cu).  Packed parameter vector: w1 [192][256],
 // b1 [256], w2 [256][256], b2 [256], w3 [256], b3 [1].

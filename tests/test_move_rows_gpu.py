@@ -20,7 +20,7 @@ def instance(rng, lay, n_plans, n_sku, sizes=(1,)):
     orders, need = [], sum(TOURS)
     while need > 0:
         k = int(rng.choice(sizes))
-        orders.append(rng.integers(0, n_sku, k).tolist())
+        orders.append(rng.choice(n_sku, k, replace=False).tolist())
         need -= k
     plans = []
     for _ in range(n_plans):
