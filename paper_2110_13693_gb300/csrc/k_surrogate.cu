@@ -20,11 +20,13 @@ constexpr int FEAT_THREADS = 256;
 // time, each lane finding its line's order from the orders' start offsets (a
 // bitmask of order starts within the 32-line window), so all lanes gather
 // slot-map entries together whatever the orders' sizes: 342,000 tours of 60
-// lines took 350 us (now 255) with a lane walking each order line by line and a binary
+// lines took 350 us (now 225) with a lane walking each order line by line and a binary
 // search for every tour's plan.  The warp writes the tour's 192 bf16 features.
-// Row r holds tour list[r] when a list is given, else tour r.
+// Row r holds tour list[r] when a list is given, else tour r; a warp takes
+// `run` (at most 31) rows in a row, whose offsets it reads at once and whose
+// plans follow from the first one's.
 __global__ void __launch_bounds__(FEAT_THREADS) k_features(EvalArgs a, FeatConst c, const int32_t* list,
-                                                           int64_t n_rows, uint4* X) {
+                                                           int64_t n_rows, uint4* X, int run) {
     __shared__ WarpFeat ws[FEAT_THREADS / 32];
     __shared__ int s_first[FEAT_THREADS / 32][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -35,65 +37,72 @@ __global__ void __launch_bounds__(FEAT_THREADS) k_features(EvalArgs a, FeatConst
     const bool shared_map = a.slot_stride == 0;
     const bool keyed = a.line_key != nullptr;   // per-line keys precomputed (shared slotting)
     const int64_t n_warps = (int64_t)gridDim.x * (FEAT_THREADS / 32);
-    for (int64_t r = (int64_t)blockIdx.x * (FEAT_THREADS / 32) + wid; r < n_rows; r += n_warps) {
-        const int t = list ? list[r] : (int)r;
-        const int q0 = a.tour_off[t], q1 = a.tour_off[t + 1];
-        const int plan = shared_map ? 0 : warp_find_plan(a, t, lane);
-        const int32_t* map = a.slot_map + (int64_t)plan * a.slot_stride;
-        bool bad = q0 < 0 || q1 < q0 || (int64_t)q1 > a.n_seq;
-        bool over = false;
-        uint32_t n_lines = 0;
-        const int q_end = bad ? q0 : q1;
-        for (int qb = q0; qb < q_end; qb += 32) {
-            int lb = 0, cnt = 0;
-            if (qb + lane < q_end) {
-                const int o = a.order_seq[qb + lane];
-                int le = 0;
-                const bool in = (unsigned)o < (unsigned)a.n_orders;
-                if (in) {
-                    lb = a.order_off[o];
-                    le = a.order_off[o + 1];
-                }
-                if (!in || lb < 0 || le < lb || le > a.n_lines) bad = true;
-                else cnt = le - lb;
-            }
-            const int incl = warp_inclusive_scan(cnt), start = incl - cnt;
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            const unsigned nonempty = __ballot_sync(0xffffffffu, cnt > 0);
-            __syncwarp();
-            if (cnt > 0) first[__popc(nonempty & lt_mask)] = lb - start;
-            __syncwarp();
-            // line p belongs to the nonempty order whose start is the last one <= p
-            int before = 0;   // nonempty orders starting before this window
-            for (int p0 = 0; p0 < total; p0 += 32) {
-                const bool head = cnt > 0 && start >= p0 && start < p0 + 32;
-                const unsigned hm = __reduce_or_sync(0xffffffffu, head ? 1u << (start - p0) : 0u);
-                const int p = p0 + lane;
-                if (p < total && !bad) {
-                    const int l = first[before + __popc(hm & (lt_mask | (1u << lane))) - 1] + p;
-                    uint32_t key;
-                    if (keyed) {
-                        key = a.line_key[l];
-                    } else {
-                        const int s = a.line_sku[l];
-                        const int loc = (unsigned)s < (unsigned)a.n_sku ? map[s] : -1;
-                        key = (unsigned)loc < (unsigned)a.g.n_loc ? loc_key(a.g, loc) : KEY_BAD;
+    for (int64_t r0 = ((int64_t)blockIdx.x * (FEAT_THREADS / 32) + wid) * run; r0 < n_rows; r0 += n_warps * run) {
+        const int t0 = list ? list[r0] : (int)r0;
+        int offs = 0;   // lane i: where tour t0 + i begins
+        if (lane <= run && (list || r0 + lane <= n_rows)) offs = a.tour_off[t0 + lane];
+        int plan = shared_map ? 0 : warp_find_plan(a, t0, lane);
+        for (int i = 0; i < run && r0 + i < n_rows; ++i) {
+            const int64_t r = r0 + i;
+            if (!shared_map)
+                while (plan + 1 < a.n_plans && a.plan_tour_off[plan + 1] <= t0 + i) ++plan;
+            const int q0 = __shfl_sync(0xffffffffu, offs, i), q1 = __shfl_sync(0xffffffffu, offs, i + 1);
+            const int32_t* map = a.slot_map + (int64_t)plan * a.slot_stride;
+            bool bad = q0 < 0 || q1 < q0 || (int64_t)q1 > a.n_seq;
+            bool over = false;
+            uint32_t n_lines = 0;
+            const int q_end = bad ? q0 : q1;
+            for (int qb = q0; qb < q_end; qb += 32) {
+                int lb = 0, cnt = 0;
+                if (qb + lane < q_end) {
+                    const int o = a.order_seq[qb + lane];
+                    int le = 0;
+                    const bool in = (unsigned)o < (unsigned)a.n_orders;
+                    if (in) {
+                        lb = a.order_off[o];
+                        le = a.order_off[o + 1];
                     }
-                    if (key == KEY_BAD) {
-                        bad = true;
-                    } else {
-                        over |= !wf_insert(w, key);
-                        ++n_lines;
-                    }
+                    if (!in || lb < 0 || le < lb || le > a.n_lines) bad = true;
+                    else cnt = le - lb;
                 }
-                before += __popc(hm);
+                const int incl = warp_inclusive_scan(cnt), start = incl - cnt;
+                const int total = __shfl_sync(0xffffffffu, incl, 31);
+                const unsigned nonempty = __ballot_sync(0xffffffffu, cnt > 0);
+                __syncwarp();
+                if (cnt > 0) first[__popc(nonempty & lt_mask)] = lb - start;
+                __syncwarp();
+                // line p belongs to the nonempty order whose start is the last one <= p
+                int before = 0;   // nonempty orders starting before this window
+                for (int p0 = 0; p0 < total; p0 += 32) {
+                    const bool head = cnt > 0 && start >= p0 && start < p0 + 32;
+                    const unsigned hm = __reduce_or_sync(0xffffffffu, head ? 1u << (start - p0) : 0u);
+                    const int p = p0 + lane;
+                    if (p < total && !bad) {
+                        const int l = first[before + __popc(hm & (lt_mask | (1u << lane))) - 1] + p;
+                        uint32_t key;
+                        if (keyed) {
+                            key = a.line_key[l];
+                        } else {
+                            const int s = a.line_sku[l];
+                            const int loc = (unsigned)s < (unsigned)a.n_sku ? map[s] : -1;
+                            key = (unsigned)loc < (unsigned)a.g.n_loc ? loc_key(a.g, loc) : KEY_BAD;
+                        }
+                        if (key == KEY_BAD) {
+                            bad = true;
+                        } else {
+                            over |= !wf_insert(w, key);
+                            ++n_lines;
+                        }
+                    }
+                    before += __popc(hm);
+                }
             }
+            bad = __any_sync(0xffffffffu, bad);
+            over = __any_sync(0xffffffffu, over);
+            n_lines = __reduce_add_sync(0xffffffffu, n_lines);
+            if ((bad || over) && lane == 0) flag(a.status, bad ? WH_STATUS_BAD_ORDER : WH_STATUS_TOUR_TOO_LONG);
+            wf_finish(w, c, lane, n_lines, X + r * 24);
         }
-        bad = __any_sync(0xffffffffu, bad);
-        over = __any_sync(0xffffffffu, over);
-        n_lines = __reduce_add_sync(0xffffffffu, n_lines);
-        if ((bad || over) && lane == 0) flag(a.status, bad ? WH_STATUS_BAD_ORDER : WH_STATUS_TOUR_TOO_LONG);
-        wf_finish(w, c, lane, n_lines, X + r * 24);
     }
 }
 
@@ -140,10 +149,12 @@ cudaError_t launch_features(const EvalArgs& a, const FeatConst& c, void* X, cons
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_features, FEAT_THREADS, 0);
     if (e != cudaSuccess) return e;
     int64_t grid = (int64_t)per_sm * num_sms;
+    // four rows a warp and turn where every warp has at least eight
+    const int run = !list && n_rows >= 8 * grid * (FEAT_THREADS / 32) ? 4 : 1;
     const int64_t want = (n_rows + FEAT_THREADS / 32 - 1) / (FEAT_THREADS / 32);
     if (grid > want) grid = want;
     if (grid < 1) grid = 1;
-    k_features<<<(int)grid, FEAT_THREADS, 0, s>>>(a, c, list, n_rows, static_cast<uint4*>(X));
+    k_features<<<(int)grid, FEAT_THREADS, 0, s>>>(a, c, list, n_rows, static_cast<uint4*>(X), run);
     return cudaGetLastError();
 }
 
