@@ -459,6 +459,16 @@ __device__ __forceinline__ uint4 order_aggregate(const EvalArgs& a, int o) {
     return make_uint4((uint32_t)bits, (uint32_t)(bits >> 32), kmax, fl);
 }
 
+// The same in 8 bytes for at most 50 aisles of at most 256 slots: the aisle
+// bits in the low 50, above them the largest key (6 bits of aisle, 8 of slot;
+// all ones: an order with an invalid line or malformed offsets).
+constexpr uint32_t PACK_BITS = 0x3FFFFu, PACK_BAD = 0x3FFFu;
+
+__device__ __forceinline__ uint2 pack_aggregate(uint4 r) {
+    const uint32_t key = (r.w & 5u) ? PACK_BAD : ((r.z >> 16) << 8) | (r.z & 0xFFu);
+    return make_uint2(r.x, (key << 18) | (r.y & PACK_BITS));
+}
+
 // line keys of one instance, zeroed plan sums, plan offset checks
 __device__ __forceinline__ void prep_instance(const EvalArgs& a, uint32_t mask, int i0, int stride) {
     if (a.line_key) {
@@ -478,6 +488,8 @@ __device__ __forceinline__ void prep_instance(const EvalArgs& a, uint32_t mask, 
     }
     if (a.order_agg)
         for (int o = i0; o < a.n_orders; o += stride) a.order_agg[o] = order_aggregate(a, o);
+    if (a.order_pack)
+        for (int o = i0; o < a.n_orders; o += stride) a.order_pack[o] = pack_aggregate(order_aggregate(a, o));
     if (a.line_ord) {
         for (int o = i0; o < a.n_orders; o += stride) {
             // malformed offsets and orders of 255 lines or more: k_eval_plan
@@ -670,21 +682,54 @@ constexpr int SSHAPE_AGG_THREADS = 256;
 // S-shape only with per-order aggregates (shared slotting, <= 64 aisles):
 // a tour's pick-aisle set is the union of its orders' aisle sets and its
 // rightmost aisle's deepest pick is the largest key over its orders, so each
-// tour merges one 16-byte record per order (no per-line work).  No shared
-// memory: full occupancy hides the order-id and record loads.
-// One warp's 32-tour chunks [c_begin, c_end): each tour merges the aggregates
-// of its orders (agg(o) -> uint4), then the S-shape closed form and the
+// tour merges one record per order (no per-line work).
+//
+// 16-byte records in global memory (any layout of <= 64 aisles)
+struct AggGlobal {
+    const uint4* t;
+    uint64_t bits = 0;
+    uint32_t kmax = 0, fl = 0;
+    __device__ __forceinline__ void take(int o) {
+        const uint4 r = __ldg(t + o);
+        bits |= (uint64_t)r.x | ((uint64_t)r.y << 32);
+        kmax = (r.w & 2u) ? max(kmax, r.z) : kmax;
+        fl |= r.w;
+    }
+    __device__ __forceinline__ bool bad() const { return (fl & 5u) != 0; }
+    __device__ __forceinline__ int aisles() const { return __popcll(bits); }
+    __device__ __forceinline__ int last_aisle() const { return (int)(kmax >> 16); }
+    __device__ __forceinline__ int last_slot() const { return (int)(kmax & 0xFFFFu); }
+};
+
+// packed 8-byte records in shared memory (k_prep's order_pack)
+struct AggShared {
+    uint32_t sa;   // shared-window address of the table
+    uint32_t lo = 0, hi = 0, top = 0;
+    __device__ __forceinline__ void take(int o) {
+        uint32_t x, y;
+        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(sa + 8u * (uint32_t)o));
+        lo |= x;
+        hi |= y & PACK_BITS;
+        top = max(top, y);   // the key is in the high bits
+    }
+    __device__ __forceinline__ bool bad() const { return (top >> 18) == PACK_BAD; }
+    __device__ __forceinline__ int aisles() const { return __popc(lo) + __popc(hi); }
+    __device__ __forceinline__ int last_aisle() const { return (int)(top >> 26); }
+    __device__ __forceinline__ int last_slot() const { return (int)((top >> 18) & 0xFFu); }
+};
+
+// One warp's 32-tour chunks [c_begin, c_end): each tour merges its orders'
+// records into a fresh copy of `empty`, then the S-shape closed form and the
 // segmented plan sums.
 template <typename Agg>
-__device__ __forceinline__ void sshape_agg_chunks(const EvalArgs& a, Agg agg, int c_begin, int c_end, int lane) {
+__device__ __forceinline__ void sshape_agg_chunks(const EvalArgs& a, const Agg empty, int c_begin, int c_end, int lane) {
     const bool vec = (reinterpret_cast<uintptr_t>(a.order_seq) & 15u) == 0;
     int plan = warp_find_plan(a, c_begin * 32, lane);
     for (int c = c_begin; c < c_end; ++c) {
         const int t = c * 32 + lane;
         const bool active = t < a.n_tours;
         while (plan + 1 < a.n_plans && a.plan_tour_off[plan + 1] <= t) ++plan;
-        uint64_t bits = 0;
-        uint32_t kmax = 0, fl = 0;
+        Agg g = empty;
         bool bad = false;
         if (active) {
             const int q0 = __ldg(a.tour_off + t), q1 = __ldg(a.tour_off + t + 1);
@@ -697,10 +742,7 @@ __device__ __forceinline__ void sshape_agg_chunks(const EvalArgs& a, Agg agg, in
                         bad = true;
                         return;
                     }
-                    const uint4 r = agg(o);
-                    bits |= (uint64_t)r.x | ((uint64_t)r.y << 32);
-                    kmax = (r.w & 2u) ? max(kmax, r.z) : kmax;
-                    fl |= r.w;
+                    g.take(o);
                 };
                 // the thread's run of order ids: scalar loads up to a 16-byte
                 // boundary, then four ids per vector load (a quarter of the
@@ -720,9 +762,8 @@ __device__ __forceinline__ void sshape_agg_chunks(const EvalArgs& a, Agg agg, in
                 if (bad) flag(a.status, WH_STATUS_BAD_ORDER);
             }
         }
-        const bool ok = active && !bad && !(fl & 5u);
-        const int m = __popcll(bits);
-        const int cs = ok ? sshape_cost(a.g, m, (int)(kmax >> 16), (int)(kmax & 0xFFFFu)) : 0;
+        const bool ok = active && !bad && !g.bad();
+        const int cs = ok ? sshape_cost(a.g, g.aisles(), g.last_aisle(), g.last_slot()) : 0;
         if (active && a.tour_s) a.tour_s[t] = ok ? cs : -1;
         const int key = active ? plan : -1;
         const long long ss = segmented_sum(cs, key, lane);
@@ -732,12 +773,39 @@ __device__ __forceinline__ void sshape_agg_chunks(const EvalArgs& a, Agg agg, in
     }
 }
 
-
 __global__ void __launch_bounds__(SSHAPE_AGG_THREADS) k_eval_sshape_agg(EvalArgs a) {
     int c_begin, c_end;
     warp_chunk_range(a, c_begin, c_end);
     if (c_begin >= c_end) return;
-    sshape_agg_chunks(a, [&](int o) { return __ldg(a.order_agg + o); }, c_begin, c_end, threadIdx.x & 31);
+    AggGlobal empty;
+    empty.t = a.order_agg;
+    sshape_agg_chunks(a, empty, c_begin, c_end, threadIdx.x & 31);
+}
+
+// A gather of 32 random 16-byte records costs the L1 a tag and a wavefront for
+// nearly every lane; 8-byte records in shared memory cost the bank conflicts
+// of 16 lanes on 16 bank pairs, about three.  4,096 mid-size plans (830,000 tours
+// of 20 orders) 49.0 -> 39.9 us a call with k_prep.
+constexpr int SSHAPE_PACK_THREADS = 512;
+
+__global__ void __launch_bounds__(SSHAPE_PACK_THREADS, 3) k_eval_sshape_pack(EvalArgs a) {
+    extern __shared__ __align__(16) uint2 s_pack[];
+    for (int o0 = threadIdx.x; o0 < a.n_orders; o0 += 4 * SSHAPE_PACK_THREADS) {
+        uint2 r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            r[u] = o0 + u * SSHAPE_PACK_THREADS < a.n_orders ? a.order_pack[o0 + u * SSHAPE_PACK_THREADS] : make_uint2(0u, 0u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (o0 + u * SSHAPE_PACK_THREADS < a.n_orders) s_pack[o0 + u * SSHAPE_PACK_THREADS] = r[u];
+    }
+    __syncthreads();
+    int c_begin, c_end;
+    warp_chunk_range(a, c_begin, c_end);
+    if (c_begin >= c_end) return;
+    AggShared empty;
+    empty.sa = smem_addr(s_pack);
+    sshape_agg_chunks(a, empty, c_begin, c_end, threadIdx.x & 31);
 }
 
 // Persistent batch kernel: CTAs pop work items (instance, chunk range) from
@@ -1087,7 +1155,20 @@ size_t eval_batch_smem_bytes(const BatchArgs& b, const Tuning& t, bool k16) {
     return s + buffer_bytes(k16, b.max_rec, t.threads);
 }
 
+bool sshape_packs(const Geo& g, int32_t n_orders) { return g.A <= 50 && g.L <= 256 && n_orders <= SSHAPE_PACK_ORDERS; }
+
 static cudaError_t launch_sshape(const EvalArgs& a, const Tuning& t, int num_sms, cudaStream_t s, int* grid_out) {
+    if (a.order_pack) {
+        const size_t smem = sizeof(uint2) * (size_t)a.n_orders;
+        int grid = 0;
+        const int warps_needed = (a.n_tours + 31) / 32;
+        const int want = (warps_needed + SSHAPE_PACK_THREADS / 32 - 1) / (SSHAPE_PACK_THREADS / 32);
+        cudaError_t e = grid_for(k_eval_sshape_pack, SSHAPE_PACK_THREADS, smem, num_sms, want, &grid);
+        if (e != cudaSuccess) return e;
+        if (grid_out) *grid_out = grid;
+        k_eval_sshape_pack<<<grid, SSHAPE_PACK_THREADS, smem, s>>>(a);
+        return cudaGetLastError();
+    }
     if (a.order_agg) {
         int grid = 0;
         const int warps_needed = (a.n_tours + 31) / 32;
@@ -1116,7 +1197,7 @@ static cudaError_t launch_sshape(const EvalArgs& a, const Tuning& t, int num_sms
 cudaError_t launch_prep(const EvalArgs& a, cudaStream_t s) {
     int work = a.n_plans;
     if (a.line_key && a.n_lines > work) work = a.n_lines;
-    if ((a.order_agg || a.line_ord) && a.n_orders > work) work = a.n_orders;
+    if ((a.order_agg || a.order_pack || a.line_ord) && a.n_orders > work) work = a.n_orders;
     int grid = (work + 255) / 256;
     if (grid > 4096) grid = 4096;
     if (grid < 1) grid = 1;

@@ -325,7 +325,9 @@ extern "C" int wh_eval_plans(wh_layout* h, const wh_orders* orders, const wh_pla
     if (rc != WH_OK) return rc;
     char* base = static_cast<char*>(h->scratch);
     a.line_key = shared_map && !agg && o.n_lines > 0 ? reinterpret_cast<uint32_t*>(base) : nullptr;
-    a.order_agg = agg ? reinterpret_cast<uint4*>(base + key_bytes) : nullptr;
+    const bool pack = agg && wh::sshape_packs(h->g, o.n_orders);
+    a.order_agg = agg && !pack ? reinterpret_cast<uint4*>(base + key_bytes) : nullptr;
+    a.order_pack = pack ? reinterpret_cast<uint2*>(base + key_bytes) : nullptr;
     a.long_list = reinterpret_cast<int32_t*>(base + key_bytes + agg_bytes);
     uint2* long_rec = rec_bytes ? reinterpret_cast<uint2*>(base + key_bytes + agg_bytes + list_bytes) : nullptr;
     a.line_ord = ord_bytes ? reinterpret_cast<uint32_t*>(base + key_bytes + agg_bytes + list_bytes + rec_bytes) : nullptr;

@@ -66,6 +66,7 @@ struct EvalArgs {
     // k_prep (flags: 1 invalid line, 2 has lines, 4 invalid offsets); NULL
     // otherwise
     uint4* order_agg;
+    uint2* order_pack;          // the same in 8 bytes (sshape_packs), instead of order_agg
     // one CTA per plan (k_eval_plan): order << 8 | place in it of every line,
     // all ones for a line of no order, built by k_prep; NULL otherwise
     uint32_t* line_ord;
@@ -341,6 +342,10 @@ cudaError_t launch_prep_batch(const BatchArgs& b, int max_work, cudaStream_t s);
 // routing mask S-shape only on a layout of at most 2,048 aisles: the
 // sort-free S-shape kernel scores the short-tour pass (and every tour)
 bool sshape_kernel_applies(const EvalArgs& a);
+// the S-shape-only kernel takes packed per-order records (k_eval_sshape_pack):
+// order books of up to 96 KB of them, two CTAs an SM
+constexpr int32_t SSHAPE_PACK_ORDERS = 12288;
+bool sshape_packs(const Geo& g, int32_t n_orders);
 // one CTA per plan (k_eval_plan.cu) instead of one tour per thread (launch_eval_short)
 bool eval_plan_applies(const EvalArgs& a, int num_sms);
 cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s);
