@@ -516,6 +516,7 @@ __device__ __forceinline__ void prep_instance(const EvalArgs& a, uint32_t mask, 
 // ------------------------------------------------------------------ kernels
 
 __global__ void k_prep(EvalArgs a) {
+    pdl_trigger();
     const int i0 = blockIdx.x * blockDim.x + threadIdx.x;   // (lines, orders and plans by grid stride)
     if (i0 == 0) *a.long_count = 0;
     prep_instance(a, a.mask, i0, gridDim.x * blockDim.x);
@@ -547,6 +548,8 @@ __global__ void __launch_bounds__(KEY16 ? 384 : 256, 2) k_eval_short(EvalArgs a)
     unsigned char* buf_base = smem + off_b;
 
     KeySrc src = global_src(a);
+    pdl_trigger();
+    pdl_wait();
     bool check_keys = true;   // keys read from global memory: every tour checks its own
     if constexpr (SMEM_TABLES) check_keys = __syncthreads_or(stage_tables<KEY16, SHARED_MAP>(a, s_desc, s_tab, src, tid, T));
     // this warp's contiguous range of 32-tour chunks
@@ -578,6 +581,7 @@ __global__ void __launch_bounds__(256) k_eval_sshape(EvalArgs a) {
         off_b = (sizeof(uint32_t) * (size_t)a.n_orders + (SHARED_MAP ? (KEY16 ? 2 : 4) : 4) * (size_t)a.n_lines + 15) &
                 ~(size_t)15;
     uint32_t* bm = reinterpret_cast<uint32_t*>(smem + off_b) + tid;   // word w at bm[w * T]
+    pdl_wait();
     const int nw = (a.g.A + 31) >> 5;
     KeySrc src = global_src(a);
     if constexpr (SMEM_TABLES) {
@@ -774,6 +778,7 @@ __device__ __forceinline__ void sshape_agg_chunks(const EvalArgs& a, const Agg e
 }
 
 __global__ void __launch_bounds__(SSHAPE_AGG_THREADS) k_eval_sshape_agg(EvalArgs a) {
+    pdl_wait();
     int c_begin, c_end;
     warp_chunk_range(a, c_begin, c_end);
     if (c_begin >= c_end) return;
@@ -790,6 +795,7 @@ constexpr int SSHAPE_PACK_THREADS = 512;
 
 __global__ void __launch_bounds__(SSHAPE_PACK_THREADS, 3) k_eval_sshape_pack(EvalArgs a) {
     extern __shared__ __align__(16) uint2 s_pack[];
+    pdl_wait();
     for (int o0 = threadIdx.x; o0 < a.n_orders; o0 += 4 * SSHAPE_PACK_THREADS) {
         uint2 r[4];
 #pragma unroll
@@ -875,6 +881,7 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_eval_long(LongArgs L) {
     __shared__ int s_meta[LONG_WARPS][32][4];   // inst, tour, plan, record count (-1: done)
     __shared__ uint32_t s_last[LONG_WARPS][32];  // largest key of the tour
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_wait();
     const int count = min(*L.count, L.cap);
     uint32_t* kb = buf[warp];
     const bool need_rr = (L.mask & WH_ROUTE_OPTIMAL) != 0;
@@ -1097,8 +1104,7 @@ cudaError_t launch_short_t(const EvalArgs& a, const Tuning& t, size_t smem, int 
     cudaError_t e = grid_for(kern, t.threads, smem, num_sms, (warps_needed + t.threads / 32 - 1) / (t.threads / 32), &grid);
     if (e != cudaSuccess) return e;
     if (grid_out) *grid_out = grid;
-    kern<<<grid, t.threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, t.threads, smem, s, a);
 }
 
 template <bool K16, bool SH, bool SM>
@@ -1110,8 +1116,7 @@ cudaError_t launch_sshape_t(const EvalArgs& a, const Tuning& t, size_t smem, int
     cudaError_t e = grid_for(kern, t.threads, smem, num_sms, (warps_needed + t.threads / 32 - 1) / (t.threads / 32), &grid);
     if (e != cudaSuccess) return e;
     if (grid_out) *grid_out = grid;
-    kern<<<grid, t.threads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, t.threads, smem, s, a);
 }
 
 template <bool K16, bool SM, bool ID16>
@@ -1166,8 +1171,7 @@ static cudaError_t launch_sshape(const EvalArgs& a, const Tuning& t, int num_sms
         cudaError_t e = grid_for(k_eval_sshape_pack, SSHAPE_PACK_THREADS, smem, num_sms, want, &grid);
         if (e != cudaSuccess) return e;
         if (grid_out) *grid_out = grid;
-        k_eval_sshape_pack<<<grid, SSHAPE_PACK_THREADS, smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_dependent(k_eval_sshape_pack, grid, SSHAPE_PACK_THREADS, smem, s, a);
     }
     if (a.order_agg) {
         int grid = 0;
@@ -1176,8 +1180,7 @@ static cudaError_t launch_sshape(const EvalArgs& a, const Tuning& t, int num_sms
         cudaError_t e = grid_for(k_eval_sshape_agg, SSHAPE_AGG_THREADS, 0, num_sms, want, &grid);
         if (e != cudaSuccess) return e;
         if (grid_out) *grid_out = grid;
-        k_eval_sshape_agg<<<grid, SSHAPE_AGG_THREADS, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_dependent(k_eval_sshape_agg, grid, SSHAPE_AGG_THREADS, 0, s, a);
     }
     const bool shared_map = a.slot_stride == 0;
     const bool k16 = t.key16 && key16_ok(a.g);
@@ -1276,8 +1279,7 @@ cudaError_t launch_eval_long(const LongArgs& L, bool shared_map, int num_sms, cu
     auto kern = shared_map ? k_eval_long<true> : k_eval_long<false>;
     const int per_sm = long_per_sm();
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    kern<<<num_sms * per_sm, LONG_WARPS * 32, 0, s>>>(L);
-    return cudaGetLastError();
+    return launch_dependent(kern, num_sms * per_sm, LONG_WARPS * 32, 0, s, L);
 }
 
 

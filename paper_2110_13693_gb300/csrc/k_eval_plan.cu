@@ -82,6 +82,8 @@ __global__ void __launch_bounds__(PL_THREADS, PL_CTAS) k_eval_plan(EvalArgs a) {
     const bool need_rr = (a.mask & WH_ROUTE_OPTIMAL) != 0;
     const bool want_s = (a.mask & WH_ROUTE_SSHAPE) != 0;
 
+    pdl_trigger();
+    pdl_wait();
     // line counts; an order book with malformed offsets or an order of 255
     // lines or more has no line -> order table to go by
     bool odd = false;
@@ -306,8 +308,7 @@ cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int grid = a.n_plans < per_sm * num_sms ? a.n_plans : per_sm * num_sms;
-    kern<<<grid, PL_THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, PL_THREADS, smem, s, a);
 }
 
 }  // namespace wh

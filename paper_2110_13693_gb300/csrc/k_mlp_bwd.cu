@@ -61,6 +61,8 @@ __global__ void __launch_bounds__(BT_THREADS) k_bwd_tail(BwdArgs b) {
     __shared__ __align__(16) __nv_bfloat16 s_t[256][BT_ROWS + 8];
     const int tid = threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * BT_ROWS;
+    pdl_trigger();
+    pdl_wait();
     if (blockIdx.y == 1) {
         // H1 transposed (the forward's activations; rows past n are zero)
         const int j = tid;
@@ -187,6 +189,8 @@ __global__ void __launch_bounds__(D1_THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_trigger();
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -323,6 +327,8 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_trigger();
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -415,12 +421,18 @@ __device__ __forceinline__ float sum_parts(const float* p, int64_t step, int cou
 // describe).  Block 0 also sums the loss.
 __global__ void k_adam_parts(BwdArgs b, float* p, float* mo, float* ve, float* G, float lr, float b1, float b2,
                              float eps, float c1, float c2, __nv_bfloat16* w1b, __nv_bfloat16* w2b,
-                             __nv_bfloat16* w1t, __nv_bfloat16* w2t, float* loss) {
+                             __nv_bfloat16* w1t, __nv_bfloat16* w2t, float* loss, float* loss_out) {
+    pdl_trigger();
+    pdl_wait();
     const int S = b.splits;
     const int nbt = (int)((b.n + BT_ROWS - 1) / BT_ROWS);
     const float* pw2 = b.part_w;                            // [S][256][256]
     const float* pw1 = b.part_w + (int64_t)S * 65536;       // [S][256][256], row 192 = b1
-    if (blockIdx.x == 0 && threadIdx.x == 0 && loss) *loss = sum_parts(b.part_t + 513, BT_PART, nbt);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const float l = sum_parts(b.part_t + 513, BT_PART, nbt);
+        *loss = l;
+        if (loss_out) *loss_out = l;
+    }
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < MLP_NPARAM;
          i += (int64_t)gridDim.x * blockDim.x) {
         float gi;
@@ -458,30 +470,26 @@ cudaError_t launch_bwd(const BwdArgs& b, const CUtensorMap& mdz2, const CUtensor
                        cudaStream_t s) {
     if (b.n <= 0) return cudaSuccess;
     const int64_t nbt = (b.n + BT_ROWS - 1) / BT_ROWS;
-    k_bwd_tail<<<dim3((unsigned)nbt, 3), BT_THREADS, 0, s>>>(b);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(k_bwd_tail, dim3((unsigned)nbt, 3), BT_THREADS, 0, s, b);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_mlp_dz1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D1_SMEM);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (b.n + 127) / 128;
-    k_mlp_dz1<<<(unsigned)(tiles < num_sms ? tiles : num_sms), D1_THREADS, D1_SMEM, s>>>(mdz2, mw2, b);
-    e = cudaGetLastError();
+    e = launch_dependent(k_mlp_dz1, (unsigned)(tiles < num_sms ? tiles : num_sms), D1_THREADS, D1_SMEM, s, mdz2, mw2, b);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM);
     if (e != cudaSuccess) return e;
-    k_mlp_wgrad<<<(unsigned)(4 * b.splits), BW_THREADS, WG_SMEM, s>>>(mh1t, mdz2t, mxt, mdz1t, b);
-    return cudaGetLastError();
+    return launch_dependent(k_mlp_wgrad, (unsigned)(4 * b.splits), BW_THREADS, WG_SMEM, s, mh1t, mdz2t, mxt, mdz1t, b);
 }
 
 cudaError_t launch_adam_parts(const BwdArgs& b, float* p, float* m, float* v, float* G, float lr, int step, void* w1b,
-                              void* w2b, void* w1t, void* w2t, float* loss, cudaStream_t s) {
+                              void* w2b, void* w1t, void* w2t, float* loss, float* loss_out, cudaStream_t s) {
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
     const int blocks = (int)((MLP_NPARAM + 255) / 256);
-    k_adam_parts<<<blocks, 256, 0, s>>>(b, p, m, v, G, lr, b1, b2, 1e-8f, c1, c2, static_cast<__nv_bfloat16*>(w1b),
-                                        static_cast<__nv_bfloat16*>(w2b), static_cast<__nv_bfloat16*>(w1t),
-                                        static_cast<__nv_bfloat16*>(w2t), loss);
-    return cudaGetLastError();
+    return launch_dependent(k_adam_parts, blocks, 256, 0, s, b, p, m, v, G, lr, b1, b2, 1e-8f, c1, c2,
+                            static_cast<__nv_bfloat16*>(w1b), static_cast<__nv_bfloat16*>(w2b),
+                            static_cast<__nv_bfloat16*>(w1t), static_cast<__nv_bfloat16*>(w2t), loss, loss_out);
 }
 
 }  // namespace wh

@@ -98,8 +98,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n_tiles = (n + TC_ROWS - 1) / TC_ROWS;
 
-    for (int i = threadIdx.x; i < 768; i += TC_THREADS)
-        par[i] = i < 256 ? P[MLP_B1_OFF + i] : i < 512 ? P[MLP_B2_OFF + i - 256] : P[MLP_W3_OFF + i - 512];
+    if (SAVE) pdl_trigger();
     if (threadIdx.x == 0) {
         *abort = 0;
         mbar_init(x_full, 1);
@@ -121,6 +120,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (SAVE) pdl_wait();
+    for (int i = threadIdx.x; i < 768; i += TC_THREADS)
+        par[i] = i < 256 ? P[MLP_B1_OFF + i] : i < 512 ? P[MLP_B2_OFF + i - 256] : P[MLP_W3_OFF + i - 512];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -364,6 +366,7 @@ cudaError_t launch_mlp_tc(const CUtensorMap& mx, const CUtensorMap& mw1, const C
     TcFault fault;
     fault.skip_tile = skip_tile;
     fault.wait_ns = wait_ns ? wait_ns : WAIT_NS;
+    if (save_acts) return launch_dependent(kern, grid, TC_THREADS, TC_SMEM, s, mx, mw1, mw2, P, n, y, status, save, fault);
     kern<<<grid, TC_THREADS, TC_SMEM, s>>>(mx, mw1, mw2, P, n, y, status, save, fault);
     return cudaGetLastError();
 }

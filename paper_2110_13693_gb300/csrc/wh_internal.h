@@ -14,6 +14,31 @@ namespace wh {
 constexpr uint32_t KEY_NONE = 0xFFFFFFFFu;
 constexpr int SHORT_MAX = 64;   // tours up to this many lines run one per thread
 
+// Programmatic dependent launch: a kernel launched by launch_dependent starts
+// as soon as every CTA of the kernel before it on the stream has called
+// pdl_trigger (or ended), and runs its prologue beside that kernel's tail;
+// pdl_wait returns once the kernels before it have completed and their writes
+// are visible, so it comes before anything they wrote is read and before
+// anything they read is written.  A kernel launched the ordinary way passes
+// both at once.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 struct Geo {
     int32_t A, L, P, S, W;
     int32_t h;      // W/2: depth of slot 0
@@ -300,7 +325,7 @@ cudaError_t launch_bwd(const BwdArgs& b, const CUtensorMap& mdz2, const CUtensor
                        const CUtensorMap& mdz2t, const CUtensorMap& mxt, const CUtensorMap& mdz1t, int num_sms,
                        cudaStream_t s);
 cudaError_t launch_adam_parts(const BwdArgs& b, float* p, float* m, float* v, float* G, float lr, int step, void* w1b,
-                              void* w2b, void* w1t, void* w2t, float* loss, cudaStream_t s);
+                              void* w2b, void* w1t, void* w2t, float* loss, float* loss_out, cudaStream_t s);
 
 struct FeatConst {
     int32_t A, L;

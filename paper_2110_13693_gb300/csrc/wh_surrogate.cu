@@ -332,9 +332,7 @@ extern "C" int wh_surrogate_train_step(wh_surrogate* s, const uint16_t* X, const
     s->last_n = n;
     s->step += 1;
     if (wh::launch_adam_parts(b, s->P, s->Mo, s->Ve, s->G, lr, s->step, s->w1b, s->w2b, s->w1t, s->w2t, s->loss,
-                              st) != cudaSuccess)
-        return WH_ECUDA;
-    if (loss_out && cudaMemcpyAsync(loss_out, s->loss, sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+                              loss_out, st) != cudaSuccess)
         return WH_ECUDA;
     return WH_OK;
 }
