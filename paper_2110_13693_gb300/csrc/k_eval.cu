@@ -29,6 +29,7 @@
 // without picks is crossed in one step (every class keeps to the cheapest
 // horizontal edge pattern it can use there), so the DP costs one step per
 // aisle that holds a pick instead of one per aisle up to the rightmost pick.
+#include <atomic>
 #include <type_traits>
 
 #include "tour_core.cuh"
@@ -1084,6 +1085,12 @@ template <typename K>
 cudaError_t grid_for(K kern, int threads, size_t smem, int num_sms, int want, int* grid) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    // at most a block an SM: no need to ask how many fit (the smallest calls
+    // are bound by the host's part of them)
+    if (want <= num_sms) {
+        *grid = want < 1 ? 1 : want;
+        return cudaSuccess;
+    }
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (e != cudaSuccess) return e;
@@ -1257,16 +1264,22 @@ cudaError_t launch_eval_batch(const BatchArgs& b, const Tuning& t, bool k16, int
 }
 
 // CTAs per SM of the long-tour kernel, the larger of its two forms: its grid
-// (and its record scratch) is sized by this
+// (and its record scratch) is sized by this.  A property of the code and the
+// architecture, asked for once (every evaluation needs it twice).
 static int long_per_sm() {
+    static std::atomic<int> known{0};
+    int m = known.load(std::memory_order_relaxed);
+    if (m > 0) return m;
     int a = 0, b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_eval_long<true>, LONG_WARPS * 32, 0) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_eval_long<false>, LONG_WARPS * 32, 0) != cudaSuccess) {
         cudaGetLastError();
         return -1;
     }
-    const int m = a > b ? a : b;
-    return m > 0 ? m : 1;
+    m = a > b ? a : b;
+    m = m > 0 ? m : 1;
+    known.store(m, std::memory_order_relaxed);
+    return m;
 }
 
 size_t long_rec_bytes(int num_sms) {
