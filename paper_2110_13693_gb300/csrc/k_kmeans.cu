@@ -23,9 +23,9 @@
 // run over the list of ordered SKUs and count the others.
 //
 // What bounds it: latency.  Paper scale (50,000 SKUs, k = 256, 20 rounds):
-// 1.16 ms a call, against 4.79 ms with a launch per seed over all SKUs (2.5 ms),
+// 1.01 ms a call, against 4.79 ms with a launch per seed over all SKUs (2.5 ms),
 // Lloyd rounds over all SKUs (1.3 ms) and the zones' ranks found by counting
-// pairs (0.65 ms): seeding 0.55 ms, Lloyd rounds 0.43, features and zones 0.1.
+// pairs (0.65 ms): seeding 0.55 ms, Lloyd rounds 0.3, features and zones 0.1.
 #include <cooperative_groups.h>
 
 #include "tour_core.cuh"
@@ -495,8 +495,10 @@ __device__ __forceinline__ int32_t dist_less_norm(const int32_t (&x)[KM_DIM], co
 // can hold most rows, and a row's 32 atomics on it would all meet in one
 // line).  Block 0 adds the never-ordered SKUs to their cluster's count; after
 // the final assignment the last block to finish (an atomic ticket, no wait)
-// ranks the clusters by weight.  21 us a round with the update at paper
-// scale (k = 256); over all SKUs, one thread a row, it took 66.
+// ranks the clusters by weight.  15 us a round with the update at paper (21
+// before each launch was made beside the tail of the one before and blocks
+// without rows left at once),
+// k = 256; over all SKUs, one thread a row, it took 66.
 constexpr int LL_SUB = 8;
 constexpr int LL_ROWS = KM_T / LL_SUB;
 constexpr int LL_STRIDE = KM_DIM + 4;
@@ -505,16 +507,20 @@ __global__ void __launch_bounds__(KM_T) k_km_lloyd(KmArgs A, int mode) {
     extern __shared__ __align__(16) int32_t sm[];
     __shared__ int s_zero;
     __shared__ bool s_last;
-    const int K = A.k, tid = threadIdx.x, na = *A.n_active;
+    const int K = A.k, tid = threadIdx.x;
     int32_t* cent = sm;                      // [K][36]
     int32_t* cnorm = cent + K * LL_STRIDE;   // [K] |c|^2
     int32_t* pcnt = cnorm + K;               // [K] the block's members
     int32_t* psum = pcnt + K;                // [K][32] and their sums (mode 0)
-    for (int i = tid; i < K * KM_DIM; i += KM_T) {
-        cent[(i / KM_DIM) * LL_STRIDE + i % KM_DIM] = A.cent[i];
-        if (mode == 0) psum[i] = 0;
-    }
+    pdl_trigger();
+    if (mode == 0)
+        for (int i = tid; i < K * KM_DIM; i += KM_T) psum[i] = 0;
     for (int c = tid; c < K; c += KM_T) pcnt[c] = 0;
+    pdl_wait();
+    const int na = *A.n_active;
+    // the grid is sized for the most SKUs that can be ordered
+    if (mode == 0 && blockIdx.x > 0 && (int)blockIdx.x * LL_ROWS >= na) return;
+    for (int i = tid; i < K * KM_DIM; i += KM_T) cent[(i / KM_DIM) * LL_STRIDE + i % KM_DIM] = A.cent[i];
     __syncthreads();
     for (int c = tid; c < K; c += KM_T) {
         int32_t nn = 0;
@@ -606,6 +612,8 @@ __global__ void __launch_bounds__(KM_T) k_km_lloyd(KmArgs A, int mode) {
 // centroids from the member sums and counts, which are cleared for the next
 // round (a block holds whole clusters)
 __global__ void __launch_bounds__(KM_T) k_km_update(KmArgs A) {
+    pdl_trigger();
+    pdl_wait();
     const int i = blockIdx.x * KM_T + threadIdx.x;
     const bool in = i < A.k * KM_DIM;
     const long long n = in ? A.cnt[i / KM_DIM] : 0;
@@ -783,10 +791,10 @@ cudaError_t launch_kmeans(const KmArgs& A, cudaStream_t s) {
     int grid = (most + LL_ROWS - 1) / LL_ROWS;
     grid = grid < 1 ? 1 : grid > 1216 ? 1216 : grid;   // up to eight blocks an SM
     for (int it = 0; it < A.iters; ++it) {
-        k_km_lloyd<<<grid, KM_T, smem, s>>>(A, 0);
-        k_km_update<<<(K * KM_DIM + KM_T - 1) / KM_T, KM_T, 0, s>>>(A);
+        if ((e = launch_dependent(k_km_lloyd, grid, KM_T, smem, s, A, 0)) != cudaSuccess) return e;
+        if ((e = launch_dependent(k_km_update, (K * KM_DIM + KM_T - 1) / KM_T, KM_T, 0, s, A)) != cudaSuccess) return e;
     }
-    k_km_lloyd<<<grid, KM_T, smem, s>>>(A, 1);
+    if ((e = launch_dependent(k_km_lloyd, grid, KM_T, smem, s, A, 1)) != cudaSuccess) return e;
     // zones
     const int tiles = (n + RS_TILE - 1) / RS_TILE;
     int passes = 1;
