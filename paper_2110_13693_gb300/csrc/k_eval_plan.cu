@@ -22,10 +22,7 @@ namespace wh {
 namespace {
 
 constexpr int PL_THREADS = 256;
-constexpr int PL_CTAS = 3;       // per SM
 constexpr int PL_MAXN = ROW_MAXN;   // longer tours go to the long-tour pass
-constexpr int PL_LIST = 1024;    // tours of a plan taken per round
-constexpr int PL_U = PL_LIST / PL_THREADS;
 
 // Line count of tour t, its orders checked: -1 for invalid offsets or ids
 // (flagged), PL_MAXN + 1 for a tour that the long-tour pass takes.  Four
@@ -64,16 +61,18 @@ __device__ __forceinline__ long long warp_sum31(int v) {
     return ((long long)hi << 16) + lo;
 }
 
-template <bool SHARED_MAP>
-__global__ void __launch_bounds__(PL_THREADS, PL_CTAS) k_eval_plan(EvalArgs a) {
+// LIST: tours of a plan taken per round (each round translates the order book
+// anew); CTAS: per SM.
+template <bool SHARED_MAP, int LIST, int CTAS>
+__global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
+    constexpr int T = PL_THREADS, PL_U = LIST / T;
     extern __shared__ __align__(16) uint32_t rows[];   // keys, then per order: place, line count, seen bit
     __shared__ int s_bin[PL_MAXN + 1];        // tours of every line count, then their first place in the list
-    __shared__ uint16_t s_list[PL_LIST];      // the round's tours by falling line count
-    __shared__ uint16_t s_base[PL_LIST];      // their rows, by tour
-    __shared__ uint8_t s_n[PL_LIST];          // their line counts, by tour
+    __shared__ uint16_t s_list[LIST];      // the round's tours by falling line count
+    __shared__ uint16_t s_base[LIST];      // their rows, by tour
+    __shared__ uint8_t s_n[LIST];          // their line counts, by tour
     __shared__ int s_total, s_unit, s_rows, s_dup;
     const int tid = threadIdx.x, lane = tid & 31;
-    constexpr int T = PL_THREADS;
     uint32_t* s_dst32 = rows + a.n_lines;     // first place of an order's lines, 16 bits each (0xFFFF: none)
     uint16_t* s_dst = reinterpret_cast<uint16_t*>(s_dst32);
     const int n_dst = (a.n_orders + 1) >> 1, n_seen = (a.n_orders + 31) >> 5;
@@ -99,8 +98,8 @@ __global__ void __launch_bounds__(PL_THREADS, PL_CTAS) k_eval_plan(EvalArgs a) {
         const int32_t* map = SHARED_MAP ? nullptr : a.slot_map + (int64_t)plan * a.slot_stride;
         // k_prep has flagged malformed plan offsets
         const int t0 = max(a.plan_tour_off[plan], 0), t1 = min(a.plan_tour_off[plan + 1], a.n_tours);
-        for (int tb = t0; tb < t1; tb += PL_LIST) {
-            const int nt = min(PL_LIST, t1 - tb);
+        for (int tb = t0; tb < t1; tb += LIST) {
+            const int nt = min(LIST, t1 - tb);
             for (int i = tid; i <= PL_MAXN; i += T) s_bin[i] = 0;
             for (int i = tid; i < n_dst; i += T) s_dst32[i] = 0xFFFFFFFFu;
             for (int i = tid; i < n_seen; i += T) s_seen[i] = 0u;
@@ -275,16 +274,16 @@ size_t plan_smem_bytes(const EvalArgs& a) {
 
 // Measured against k_eval_short + k_eval_long (us a call, GB300; orders x
 // tours a plan x lines a tour):
-//   own slottings    4,000 x 167 x 59, 500 aisles: 16 plans 58 -> 35,
+//   own slottings    4,000 x 167 x 59, 500 aisles: 16 plans 58 -> 32,
 //                    500 plans 167 -> 68, 2,000 plans 516 -> 202
-//                    4,000 x 200 x 49, 40 aisles: 16 plans 58 -> 32,
+//                    4,000 x 200 x 49, 40 aisles: 16 plans 58 -> 28,
 //                    2,000 plans 238 -> 156
-//                    300 x 38 x 20: 500 plans 33 -> 27, 2,000 plans 40 -> 50
-//                    400 x 17 x 59: 500 plans 54 -> 38, 2,000 plans 82 -> 77
-//   shared, 32-bit   4,000 x 167 x 59: 16 plans 46 -> 33, 2,000 plans 334 -> 153
-//                    400 x 17 x 59: 152 plans 37 -> 25, 2,000 plans 50 -> 72
-//                    3,000 x 375 x 20: 64 plans 25 -> 29, 152 plans 29 -> 29,
-//                    2,000 plans 206 -> 113
+//                    300 x 38 x 20: 500 plans 33 -> 19, 2,000 plans 40 -> 50
+//                    400 x 17 x 59: 500 plans 54 -> 23, 2,000 plans 82 -> 77
+//   shared, 32-bit   4,000 x 167 x 59: 16 plans 46 -> 29, 2,000 plans 334 -> 145
+//                    400 x 17 x 59: 152 plans 37 -> 19, 2,000 plans 50 -> 72
+//                    3,000 x 375 x 20: 64 plans 25 -> 29, 152 plans 29 -> 27,
+//                    2,000 plans 206 -> 99
 // So: many plans of few tours (a CTA's threads idle, and one tour per thread
 // fills the chip anyway) and few plans of short tours under a shared slotting
 // (k_eval_short has no latency of gathers or of a long-tour pass there) stay.
@@ -298,16 +297,28 @@ bool eval_plan_applies(const EvalArgs& a, int num_sms) {
     return a.n_plans >= num_sms || (double)a.n_lines * (double)a.n_seq > 32.0 * (double)a.n_orders * (double)a.n_tours;
 }
 
+// Three CTAs an SM (60 KB an order book at paper scale; what is left of the
+// 228 KB is the L1 that the gathers go through; 320 threads a CTA took the
+// same time), or four with lists of 512 tours where four books leave that much
+// too and few plans need a second round.  At paper scale four CTAs left the L1
+// 3 KB and took 1,019 us instead of 745; 2,000 plans of 3,000 orders in 300
+// aisles 141 -> 126 us, under a shared slotting (no gathers) 113 -> 99.
 cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s) {
     const size_t smem = plan_smem_bytes(a);
-    auto kern = a.slot_stride == 0 ? k_eval_plan<true> : k_eval_plan<false>;
+    const bool shared = a.slot_stride == 0;
+    const bool four = smem <= (shared ? 53 : 40) * 1024 && a.n_tours <= 448ll * a.n_plans;
+    auto kern = shared ? (four ? k_eval_plan<true, 512, 4> : k_eval_plan<true, 1024, 3>)
+                       : (four ? k_eval_plan<false, 512, 4> : k_eval_plan<false, 1024, 3>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PL_THREADS, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const int grid = a.n_plans < per_sm * num_sms ? a.n_plans : per_sm * num_sms;
+    int grid = a.n_plans;
+    if (grid > num_sms) {
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PL_THREADS, smem);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        if (grid > per_sm * num_sms) grid = per_sm * num_sms;
+    }
     return launch_dependent(kern, grid, PL_THREADS, smem, s, a);
 }
 
