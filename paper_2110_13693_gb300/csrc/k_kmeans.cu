@@ -495,10 +495,9 @@ __device__ __forceinline__ int32_t dist_less_norm(const int32_t (&x)[KM_DIM], co
 // can hold most rows, and a row's 32 atomics on it would all meet in one
 // line).  Block 0 adds the never-ordered SKUs to their cluster's count; after
 // the final assignment the last block to finish (an atomic ticket, no wait)
-// ranks the clusters by weight.  15 us a round with the update at paper (21
-// before each launch was made beside the tail of the one before and blocks
-// without rows left at once),
-// k = 256; over all SKUs, one thread a row, it took 66.
+// ranks the clusters by weight.  15 us a round with the update at paper scale
+// (k = 256); 21 before each launch was made beside the tail of the one before
+// and blocks without rows left at once; 66 over all SKUs, one thread a row.
 constexpr int LL_SUB = 8;
 constexpr int LL_ROWS = KM_T / LL_SUB;
 constexpr int LL_STRIDE = KM_DIM + 4;
