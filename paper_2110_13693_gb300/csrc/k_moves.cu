@@ -69,6 +69,8 @@ constexpr int MVT_THREADS = 256;
 constexpr int MVT_MAX_ORDERS = 12288;   // 48 KB of shared memory
 
 __global__ void __launch_bounds__(MVT_THREADS) k_mv_tours_plan(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ int32_t s_row[];
     const EvalArgs& a = M.a;
     for (int p = blockIdx.x; p < a.n_plans; p += gridDim.x) {
@@ -120,6 +122,8 @@ __global__ void __launch_bounds__(MVT_THREADS) k_mv_tours_plan(MoveArgs M) {
 }
 
 __global__ void k_mv_sku_count(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     const EvalArgs& a = M.a;
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < a.n_lines; l += gridDim.x * blockDim.x) {
         const int s = a.line_sku[l];
@@ -134,6 +138,8 @@ __global__ void k_mv_sku_count(MoveArgs M) {
 constexpr int SKU_ALLOC_T = 1024;
 
 __global__ void __launch_bounds__(SKU_ALLOC_T) k_mv_sku_alloc(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ int warp_tot[32];
     __shared__ int s_base;
     const int n = M.a.n_sku, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -155,6 +161,8 @@ __global__ void __launch_bounds__(SKU_ALLOC_T) k_mv_sku_alloc(MoveArgs M) {
 }
 
 __global__ void k_mv_sku_fill(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     const EvalArgs& a = M.a;
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < a.n_orders; o += gridDim.x * blockDim.x) {
         int lb, le;
@@ -173,6 +181,8 @@ __global__ void k_mv_sku_fill(MoveArgs M) {
 
 // status and task count of every move; deltas zeroed
 __global__ void k_mv_count(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     const EvalArgs& a = M.a;
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M.n_moves; m += gridDim.x * blockDim.x) {
         const int4 mv = M.moves[m];
@@ -271,6 +281,8 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long* war
 }
 
 __global__ void k_scan_blocks(int64_t* v, int64_t n, int64_t* block_tot) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ long long wt[32];
     const int64_t i = (int64_t)blockIdx.x * SCAN_T + threadIdx.x;
     const long long x = i < n ? v[i] : 0;
@@ -281,6 +293,8 @@ __global__ void k_scan_blocks(int64_t* v, int64_t n, int64_t* block_tot) {
 }
 
 __global__ void k_scan_top(int64_t* block_tot, int nb) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ long long wt[32];
     __shared__ long long carry;
     if (threadIdx.x == 0) carry = 0;
@@ -299,6 +313,8 @@ __global__ void k_scan_top(int64_t* block_tot, int nb) {
 }
 
 __global__ void k_scan_add(int64_t* v, int64_t n, const int64_t* block_tot) {
+    pdl_trigger();
+    pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * SCAN_T + threadIdx.x;
     if (i < n) v[i] += block_tot[blockIdx.x];
 }
@@ -312,6 +328,8 @@ __global__ void k_scan_add(int64_t* v, int64_t n, const int64_t* block_tot) {
 constexpr int MVF_SERIAL = 8;
 
 __global__ void k_mv_fill(MoveArgs M, int unit) {
+    pdl_trigger();
+    pdl_wait();
     const EvalArgs& a = M.a;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -362,9 +380,15 @@ __global__ void k_mv_fill(MoveArgs M, int unit) {
                 const int k0 = __shfl_sync(0xffffffffu, lk[side], src), mm = __shfl_sync(0xffffffffu, m, src);
                 const int64_t r = __shfl_sync(0xffffffffu, row, src);
                 int4* out = M.tasks + __shfl_sync(0xffffffffu, t0, src) + k0;
-                for (int i = lane; i < n; i += 32) {
-                    const int o = M.sku_orders[b + i];
-                    out[i] = make_int4(mm, M.order_tour[r + o], o, side ? -3 : -2);
+                for (int i0 = lane; i0 < n; i0 += 128) {   // four entries a lane in flight
+                    int o[4], t[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) o[u] = i0 + 32 * u < n ? M.sku_orders[b + i0 + 32 * u] : 0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) t[u] = i0 + 32 * u < n ? M.order_tour[r + o[u]] : 0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (i0 + 32 * u < n) out[i0 + 32 * u] = make_int4(mm, t[u], o[u], side ? -3 : -2);
                 }
             }
         }
@@ -568,6 +592,8 @@ __device__ __forceinline__ void mv_long_commit(const MoveArgs& M, int64_t i, int
 }
 
 __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ uint32_t buf[LONG_WARPS][LONG_MAXL];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int count = min(*M.long_count, M.long_cap);
@@ -656,6 +682,8 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
 }
 
 __global__ void k_mv_long_dp(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     const int count = min(min(*M.long_count, M.long_cap), M.long_rec_cap);
     for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < count; w += gridDim.x * blockDim.x) {
         const int m = M.long_m[w];
@@ -668,6 +696,8 @@ __global__ void k_mv_long_dp(MoveArgs M) {
 
 // moves that ended with a non-zero status report zero deltas
 __global__ void k_mv_finish(MoveArgs M) {
+    pdl_trigger();
+    pdl_wait();
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M.n_moves; m += gridDim.x * blockDim.x) {
         if (M.mstatus[m] != 0) {
             M.delta[2 * m] = 0;
@@ -697,18 +727,24 @@ __global__ void k_occupancy(const int32_t* slot_map, int64_t stride, int32_t n_p
 
 }  // namespace
 
+// The moves' short kernels, a dozen in a row: each waits for the one before it
+// as its first statement (pdl_wait) and is launched beside its tail.  The two
+// large ones (k_mv_eval, k_task_features) are launched the ordinary way and
+// trigger nothing early: beside another kernel's blocks they start with that
+// kernel's split of L1 and shared memory, and later blocks would take theirs
+// (the plain step 635 us instead of 574).
 cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s, bool reuse_index) {
     const EvalArgs& a = M.a;
     if (reuse_index) {
         // the order -> tour table, the tours' line counts and the SKU ->
         // orders index of the same plans are in place: only the moves' checks,
         // task counts and their scan
-        k_mv_count<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
+        launch_dependent(k_mv_count, grid_of(M.n_moves, 256), 256, 0, s, M);
         const int64_t n = (int64_t)M.n_moves + 1;
         const int nb = (int)((n + SCAN_T - 1) / SCAN_T);
-        k_scan_blocks<<<nb, SCAN_T, 0, s>>>(M.task_off, n, M.scan_aux);
-        k_scan_top<<<1, SCAN_T, 0, s>>>(M.scan_aux, nb);
-        k_scan_add<<<nb, SCAN_T, 0, s>>>(M.task_off, n, M.scan_aux);
+        launch_dependent(k_scan_blocks, nb, SCAN_T, 0, s, M.task_off, n, M.scan_aux);
+        launch_dependent(k_scan_top, 1, SCAN_T, 0, s, M.scan_aux, nb);
+        launch_dependent(k_scan_add, nb, SCAN_T, 0, s, M.task_off, n, M.scan_aux);
         return cudaGetLastError();
     }
     const bool per_plan = a.n_orders <= MVT_MAX_ORDERS;
@@ -727,16 +763,16 @@ cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s,
     } else if (a.n_tours > 0) {
         k_mv_tours<<<grid_of(a.n_tours, 256), 256, 0, s>>>(M);
     }
-    if (a.n_lines > 0) k_mv_sku_count<<<grid_of(a.n_lines, 256), 256, 0, s>>>(M);
-    if (a.n_sku > 0) k_mv_sku_alloc<<<(a.n_sku + SKU_ALLOC_T - 1) / SKU_ALLOC_T, SKU_ALLOC_T, 0, s>>>(M);
-    if (a.n_orders > 0) k_mv_sku_fill<<<grid_of(a.n_orders, 256), 256, 0, s>>>(M);
-    k_mv_count<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
+    if (a.n_lines > 0) launch_dependent(k_mv_sku_count, grid_of(a.n_lines, 256), 256, 0, s, M);
+    if (a.n_sku > 0) launch_dependent(k_mv_sku_alloc, (a.n_sku + SKU_ALLOC_T - 1) / SKU_ALLOC_T, SKU_ALLOC_T, 0, s, M);
+    if (a.n_orders > 0) launch_dependent(k_mv_sku_fill, grid_of(a.n_orders, 256), 256, 0, s, M);
+    launch_dependent(k_mv_count, grid_of(M.n_moves, 256), 256, 0, s, M);
     // exclusive scan of n_moves + 1 task counts
     const int64_t n = (int64_t)M.n_moves + 1;
     const int nb = (int)((n + SCAN_T - 1) / SCAN_T);
-    k_scan_blocks<<<nb, SCAN_T, 0, s>>>(M.task_off, n, M.scan_aux);
-    k_scan_top<<<1, SCAN_T, 0, s>>>(M.scan_aux, nb);
-    k_scan_add<<<nb, SCAN_T, 0, s>>>(M.task_off, n, M.scan_aux);
+    launch_dependent(k_scan_blocks, nb, SCAN_T, 0, s, M.task_off, n, M.scan_aux);
+    launch_dependent(k_scan_top, 1, SCAN_T, 0, s, M.scan_aux, nb);
+    launch_dependent(k_scan_add, nb, SCAN_T, 0, s, M.task_off, n, M.scan_aux);
     return cudaGetLastError();
 }
 
@@ -746,7 +782,7 @@ cudaError_t launch_moves_fill(const MoveArgs& M, int num_sms, cudaStream_t s) {
     if (M.n_moves <= 0) return cudaSuccess;
     const int64_t warps = (int64_t)num_sms * 32, u = (M.n_moves + warps - 1) / warps;
     const int unit = u > 32 ? 32 : (int)u;
-    k_mv_fill<<<grid_of((M.n_moves + unit - 1) / unit * 32, 256), 256, 0, s>>>(M, unit);
+    launch_dependent(k_mv_fill, grid_of((M.n_moves + unit - 1) / unit * 32, 256), 256, 0, s, M, unit);
     return cudaGetLastError();
 }
 
@@ -770,10 +806,10 @@ cudaError_t launch_moves_long(const MoveArgs& M, int num_sms, cudaStream_t s) {
         int per_sm = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_long_rec, LONG_WARPS * 32, 0);
         if (e != cudaSuccess) return e;
-        k_mv_long_rec<<<num_sms * (per_sm > 0 ? per_sm : 1), LONG_WARPS * 32, 0, s>>>(M);
-        k_mv_long_dp<<<grid_of(M.long_rec_cap, 128), 128, 0, s>>>(M);
+        launch_dependent(k_mv_long_rec, num_sms * (per_sm > 0 ? per_sm : 1), LONG_WARPS * 32, 0, s, M);
+        launch_dependent(k_mv_long_dp, grid_of(M.long_rec_cap, 128), 128, 0, s, M);
     }
-    if (M.n_moves > 0) k_mv_finish<<<grid_of(M.n_moves, 256), 256, 0, s>>>(M);
+    if (M.n_moves > 0) launch_dependent(k_mv_finish, grid_of(M.n_moves, 256), 256, 0, s, M);
     return cudaGetLastError();
 }
 
@@ -786,6 +822,8 @@ namespace {
 // One CTA per plan: the move with the most negative optimal-cost delta among
 // the plan's moves of status 0 (ties: lowest index) is applied in place.
 __global__ void k_ls_apply(LsArgs L) {
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ int32_t seg[];
     __shared__ long long s_best;
     __shared__ int s_pos[2];
@@ -1005,9 +1043,11 @@ __global__ void __launch_bounds__(TF_THREADS) k_task_features(MoveArgs M, FeatCo
 // Predicted delta of every move (sum over its counted tasks, in order), then
 // per plan the `keep` moves with the lowest predicted delta (ties: lowest
 // index); unfilled places get an invalid move that scores status 3.
-constexpr int SCORE_SERIAL = 32;
+constexpr int SCORE_SERIAL = 12;
 
 __global__ void k_screen_score(ScreenArgs S) {
+    pdl_trigger();
+    pdl_wait();
     const MoveArgs& M = S.M;
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1079,6 +1119,8 @@ __global__ void k_screen_score(ScreenArgs S) {
 }
 
 __global__ void k_screen_select(ScreenArgs S) {
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int n_plans = S.M.a.n_plans;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -1124,8 +1166,8 @@ cudaError_t launch_task_features(const MoveArgs& M, const FeatConst& c, void* X,
 }
 
 cudaError_t launch_screen_select(const ScreenArgs& S, cudaStream_t s) {
-    k_screen_score<<<grid_of(S.M.n_moves, 256), 256, 0, s>>>(S);
-    k_screen_select<<<grid_of((int64_t)S.M.a.n_plans * 32, 256), 256, 0, s>>>(S);
+    launch_dependent(k_screen_score, grid_of(S.M.n_moves, 256), 256, 0, s, S);
+    launch_dependent(k_screen_select, grid_of((int64_t)S.M.a.n_plans * 32, 256), 256, 0, s, S);
     return cudaGetLastError();
 }
 
@@ -1135,7 +1177,7 @@ cudaError_t launch_ls_apply(const LsArgs& L, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     int grid = L.a.n_plans < 65536 ? L.a.n_plans : 65536;
     if (grid < 1) grid = 1;
-    k_ls_apply<<<grid, 256, smem, s>>>(L);
+    launch_dependent(k_ls_apply, grid, 256, smem, s, L);
     return cudaGetLastError();
 }
 
