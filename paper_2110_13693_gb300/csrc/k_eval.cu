@@ -11,8 +11,8 @@
 //   k_eval_short  -- one tour per thread for tours of <= 64 lines.  A warp
 //                    owns 32 consecutive tours; keys are gathered from the
 //                    shared-memory order book into registers and sorted by a
-//                    fully unrolled bitonic network (two 16-bit keys per
-//                    register when the layout allows, so one min/max pair
+//                    fully unrolled network (merge exchange; two 16-bit keys
+//                    per register when the layout allows, so one min/max pair
 //                    serves two comparators), reduced to per-aisle records
 //                    (aisle, shallowest and deepest pick, largest gap between
 //                    consecutive picks) in shared memory, then the S-shape
@@ -22,6 +22,8 @@
 //                    after the table staging.
 //   k_eval_long   -- one warp per tour for longer tours: shared-memory
 //                    bitonic sort, then one lane runs the record scan and DP.
+//   k_eval_sshape*   the S-shape rule alone, without a sort.
+//   (k_eval_plan.cu: one CTA per plan, for own slottings and 32-bit keys)
 //
 // The optimal-route DP is the Ratliff-Rosenthal programme in a reduced form:
 // the depot is a_0 itself (start state "a_0 in the tour, even degree"), the
