@@ -1035,7 +1035,7 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_eval_long(LongArgs L) {
                 }
             }
             if (lane == 0) {
-                const uint32_t kl = kb[n - 1];   // rightmost aisle, its deepest slot
+                const uint32_t kl = n > 0 ? kb[n - 1] : 0u;   // rightmost aisle, its deepest slot
                 if (rec && m <= LONG_RMAX) {
                     s_meta[warp][j][0] = inst;
                     s_meta[warp][j][1] = t;
