@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
     __shared__ uint16_t s_base[LIST];      // their rows, by tour
     __shared__ uint8_t s_n[LIST];          // their line counts, by tour
     __shared__ int s_total, s_unit, s_rows, s_dup;
+    __shared__ bool s_untidy;
     const int tid = threadIdx.x, lane = tid & 31;
     uint32_t* s_dst32 = rows + a.n_lines;     // first place of an order's lines, 16 bits each (0xFFFF: none)
     uint16_t* s_dst = reinterpret_cast<uint16_t*>(s_dst32);
@@ -93,12 +94,23 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
         s_cnt[o] = ok ? (uint8_t)(le - lb) : 0;
         odd |= !ok;
     }
+    if (tid == 0) s_untidy = (__ldcg(a.status) & WH_STATUS_BAD_OFFSET) != 0;
     odd = __syncthreads_or(odd);
 
+    // Malformed plan offsets (k_prep has flagged them; or another call whose
+    // bit nobody has read) must still leave every tour with one plan, the first
+    // that ends behind it or else the last, as k_eval_short has it: a plan
+    // begins at the largest end of those before.
+    const bool untidy = s_untidy;
+    int begin = 0, seen = 0;   // the largest of plan offsets 1 .. seen - 1
     for (int plan = blockIdx.x; plan < a.n_plans; plan += gridDim.x) {
         const int32_t* map = SHARED_MAP ? nullptr : a.slot_map + (int64_t)plan * a.slot_stride;
-        // k_prep has flagged malformed plan offsets
-        const int t0 = max(a.plan_tour_off[plan], 0), t1 = min(a.plan_tour_off[plan + 1], a.n_tours);
+        int t0 = a.plan_tour_off[plan], t1 = a.plan_tour_off[plan + 1];
+        if (untidy) {
+            for (; seen <= plan; ++seen) begin = max(begin, seen > 0 ? a.plan_tour_off[seen] : 0);
+            t0 = min(begin, a.n_tours);
+            t1 = plan == a.n_plans - 1 ? a.n_tours : min(max(begin, t1), a.n_tours);
+        }
         for (int tb = t0; tb < t1; tb += LIST) {
             const int nt = min(LIST, t1 - tb);
             for (int i = tid; i <= PL_MAXN; i += T) s_bin[i] = 0;
