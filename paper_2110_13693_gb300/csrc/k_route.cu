@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(RT_WARPS * 32) k_routes(EvalArgs a, const int3
         ok = cls == C_E0;   // the walk starts at the depot, on the front
         if (h_back((int)(W.dec[0] >> (6 * W.cls[0])) & 7) != 0) ok = 0;
     }
+    __syncwarp();   // lane 0's classes are read by every lane (a shuffle orders no memory)
     ok = __shfl_sync(0xffffffffu, ok, 0);
     if (!ok) return fail(WH_STATUS_BAD_OFFSET);
     // per pick aisle, the edges into it from the left (front, back: 0..2 each)
