@@ -710,14 +710,13 @@ struct AggGlobal {
 
 // packed 8-byte records in shared memory (k_prep's order_pack)
 struct AggShared {
-    uint32_t sa;   // shared-window address of the table
+    const uint2* t;
     uint32_t lo = 0, hi = 0, top = 0;
     __device__ __forceinline__ void take(int o) {
-        uint32_t x, y;
-        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(sa + 8u * (uint32_t)o));
-        lo |= x;
-        hi |= y & PACK_BITS;
-        top = max(top, y);   // the key is in the high bits
+        const uint2 r = t[o];
+        lo |= r.x;
+        hi |= r.y & PACK_BITS;
+        top = max(top, r.y);   // the key is in the high bits
     }
     __device__ __forceinline__ bool bad() const { return (top >> 18) == PACK_BAD; }
     __device__ __forceinline__ int aisles() const { return __popc(lo) + __popc(hi); }
@@ -813,7 +812,7 @@ __global__ void __launch_bounds__(SSHAPE_PACK_THREADS, 3) k_eval_sshape_pack(Eva
     warp_chunk_range(a, c_begin, c_end);
     if (c_begin >= c_end) return;
     AggShared empty;
-    empty.sa = smem_addr(s_pack);
+    empty.t = s_pack;
     sshape_agg_chunks(a, empty, c_begin, c_end, threadIdx.x & 31);
 }
 
