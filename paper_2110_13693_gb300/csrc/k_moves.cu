@@ -160,21 +160,64 @@ __global__ void __launch_bounds__(SKU_ALLOC_T) k_mv_sku_alloc(MoveArgs M) {
     }
 }
 
+// Every order once in the list of each of its SKUs, also where the SKU is on
+// several of its lines: a line is skipped when one before it has its SKU.  A
+// lane looks back over the lines of its own order up to MVS_SERIAL lines, four
+// lines' SKUs and then their places in flight; a longer order is taken by the
+// whole warp, 32 lines at a time.
+constexpr int MVS_SERIAL = 32;
+
 __global__ void k_mv_sku_fill(MoveArgs M) {
     pdl_trigger();
     pdl_wait();
     const EvalArgs& a = M.a;
-    for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < a.n_orders; o += gridDim.x * blockDim.x) {
-        int lb, le;
-        if (order_lines_checked(a, o, lb, le) < 0) continue;
-        for (int l = lb; l < le; ++l) {
-            const int s = a.line_sku[l];
-            if ((unsigned)s >= (unsigned)a.n_sku) continue;
-            // (orders with malformed, overlapping line ranges hold more lines
-            // than there are)
-            const int k = M.sku_off[s] + atomicAdd(&M.sku_cur[s], 1);
-            if (k < a.n_lines) M.sku_orders[k] = o;
-            else atomicSub(&M.sku_cur[s], 1);
+    const int lane = threadIdx.x & 31;
+    auto place = [&](int s) { return M.sku_off[s] + atomicAdd(&M.sku_cur[s], 1); };
+    auto put = [&](int s, int o, int k) {
+        // (orders with malformed, overlapping line ranges hold more lines
+        // than there are)
+        if (k < a.n_lines) M.sku_orders[k] = o;
+        else atomicSub(&M.sku_cur[s], 1);
+    };
+    for (int o0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); o0 < a.n_orders; o0 += gridDim.x * blockDim.x) {
+        const int o = o0 + lane;
+        int lb = 0, le = 0;
+        if (o < a.n_orders && order_lines_checked(a, o, lb, le) < 0) lb = le = 0;
+        const bool lng = le - lb > MVS_SERIAL;
+        for (int l0 = lb; !lng && l0 < le; l0 += 4) {
+            int s[4], k[4];
+            bool add[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[u] = l0 + u < le ? a.line_sku[l0 + u] : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                add[u] = (unsigned)s[u] < (unsigned)a.n_sku;
+#pragma unroll
+                for (int v = 0; v < u; ++v) add[u] &= s[v] != s[u];
+            }
+            for (int l = lb; l < l0; ++l) {
+                const int t = a.line_sku[l];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) add[u] &= t != s[u];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) k[u] = add[u] ? place(s[u]) : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (add[u]) put(s[u], o, k[u]);
+        }
+        for (unsigned longs = __ballot_sync(0xffffffffu, lng); longs; longs &= longs - 1) {
+            const int src = __ffs(longs) - 1;
+            const int b = __shfl_sync(0xffffffffu, lb, src), e = __shfl_sync(0xffffffffu, le, src);
+            for (int l0 = b; l0 < e; l0 += 32) {
+                const int s = l0 + lane < e ? a.line_sku[l0 + lane] : -1;
+                // of equal SKUs among the 32 the first lane's line counts
+                const unsigned same = __match_any_sync(0xffffffffu, s);
+                bool add = (unsigned)s < (unsigned)a.n_sku && (same & ((1u << lane) - 1u)) == 0;
+#pragma unroll 8
+                for (int l = b; l < l0; ++l) add &= a.line_sku[l] != s;
+                if (add) put(s, o0 + src, place(s));
+            }
         }
     }
 }
