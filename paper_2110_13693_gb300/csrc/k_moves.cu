@@ -539,10 +539,15 @@ __global__ void __launch_bounds__(ROW_THREADS, 5) k_mv_eval(MoveArgs M, int unit
 }
 
 // The changed tour of task `tk` by one warp: lane j takes the changed tour's orders
-// j, j + 32, ... (the added order last) and stores their line indices at
-// positions given by a warp prefix sum of the order line counts; then the
-// lanes turn positions x, x + 32, ... into keys.  Only the first `cap`
-// positions are stored.  Returns ok and sets n and primary (all warp-uniform).
+// j, j + 32, ... (the added order last), stores their line indices at
+// positions given by a warp prefix sum of the order line counts and, for a SKU
+// move, looks for the moved SKUs on them; then, if the task is the counted one
+// of its tour, the lanes turn positions x, x + 32, ... into keys.  (A popular SKU is
+// on many of a tour's orders, and all but one of its tasks there end here.  With a
+// lane looking through the tour's orders for every line found, 16,384 moves on tours
+// of 200 lines took 1,057 us a call; now 400.)
+// Only the first `cap` positions are stored.  Returns ok and sets n and
+// primary (all warp-uniform).
 __device__ __forceinline__ bool walk_task_warp(const MoveArgs& M, const int4 tk, const int4 mv, uint32_t* kb,
                                                int cap, int lane, int& n_out, bool& primary) {
     const EvalArgs& a = M.a;
@@ -556,7 +561,7 @@ __device__ __forceinline__ bool walk_task_warp(const MoveArgs& M, const int4 tk,
     int hit_min = 0x7fffffff, n = 0;
     bool own_has_s1 = false;
     // the lines' indices at their positions in the changed tour (lanes over
-    // orders; shared stores only)
+    // orders)
     for (int qb = q0; qb < q_end; qb += 32) {
         const int q = qb + lane;
         int o = -1, lb = 0, le = 0;
@@ -568,16 +573,33 @@ __device__ __forceinline__ bool walk_task_warp(const MoveArgs& M, const int4 tk,
         const int cnt = le - lb;
         const int incl = warp_inclusive_scan(cnt);
         int pos = n + incl - cnt;
+        if (swap) {
+            for (int l0 = lb; l0 < le; l0 += 4) {
+                int sk[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) sk[u] = l0 + u < le ? a.line_sku[l0 + u] : -1;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (sk[u] < 0 || !sku_hit(sk[u], mv)) continue;
+                    hit_min = min(hit_min, o);
+                    own_has_s1 |= o == tk.z && sk[u] == mv.y;
+                }
+            }
+        }
         for (int l = lb; l < le; ++l, ++pos)
             if (pos < cap) kb[pos] = (uint32_t)l;
         n += __shfl_sync(0xffffffffu, incl, 31);
     }
     bad = __any_sync(0xffffffffu, bad);
+    hit_min = __reduce_min_sync(0xffffffffu, hit_min);
+    own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
+    primary = !swap || (hit_min == tk.z && (tk.w == -2 || !own_has_s1));
+    n_out = n;
+    if (bad || !primary) return !bad;
     __syncwarp();
     // keys: lanes over positions, four a lane with their SKU and slot loads in
-    // flight together.  A line whose SKU the move changes finds its orders
-    // among the tour's (a SKU move keeps every order of the tour)
-    const int nn = bad ? 0 : min(n, cap);
+    // flight together
+    const int nn = min(n, cap);
     for (int x0 = 0; x0 < nn; x0 += 128) {
         int l[4], sk[4], loc[4];
 #pragma unroll
@@ -597,25 +619,10 @@ __device__ __forceinline__ bool walk_task_warp(const MoveArgs& M, const int4 tk,
                 bad = true;
                 continue;
             }
-            if (swap && sku_hit(sk[u], mv)) {
-                for (int q = q0; q < q1; ++q) {
-                    const int o = a.order_seq[q];
-                    if ((unsigned)o >= (unsigned)a.n_orders) continue;
-                    if (l[u] >= a.order_off[o] && l[u] < a.order_off[o + 1]) {
-                        hit_min = min(hit_min, o);
-                        if (o == tk.z && sk[u] == mv.y) own_has_s1 = true;
-                    }
-                }
-            }
             kb[x0 + 32 * u + lane] = loc_key(a.g, loc[u]);
         }
     }
-    const bool ok = !__any_sync(0xffffffffu, bad);
-    hit_min = __reduce_min_sync(0xffffffffu, hit_min);
-    own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
-    primary = !swap || (hit_min == tk.z && (tk.w == -2 || !own_has_s1));
-    n_out = n;
-    return ok;
+    return !__any_sync(0xffffffffu, bad);
 }
 
 // Tasks of more than ROW_MAXN lines, in two kernels.  k_mv_long_rec: one
