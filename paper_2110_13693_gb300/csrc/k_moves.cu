@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 5) k_mv_eval(MoveArgs M, int unit
             flag(a.status, WH_STATUS_BAD_ORDER);
             M.mstatus[tk.x] = 3;
         }
-        if (M.stats) {   // changed tours walked and their lines (the moves' roofline); k_mv_long_rec adds its own
+        if (M.stats) {   // changed tours walked and their lines (the moves' roofline); k_mv_long adds its own
             const bool w = active && ok && !lng;
             const unsigned walked = __reduce_add_sync(0xffffffffu, w ? 1u : 0u);
             const unsigned lines = __reduce_add_sync(0xffffffffu, w ? (unsigned)n : 0u);
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 5) k_mv_eval(MoveArgs M, int unit
             ds = (long long)cs - M.tour_s_old[tk.y];
             dr = (long long)cr - M.tour_rr_old[tk.y];
         }
-        if (active && !lng)   // k_mv_long_rec and k_mv_long_dp write the long ones
+        if (active && !lng)   // k_mv_long writes the long ones
             M.task_cost[i] = run ? make_int2(cs, cr) : make_int2(-1, -1);
         const int key = active ? tk.x : -1;
         const long long ss = segmented_sum(ds, key, lane);
@@ -625,13 +625,15 @@ __device__ __forceinline__ bool walk_task_warp(const MoveArgs& M, const int4 tk,
     return !__any_sync(0xffffffffu, bad);
 }
 
-// Tasks of more than ROW_MAXN lines, in two kernels.  k_mv_long_rec: one
-// warp per task walks the changed tour (walk_task_warp), sorts its keys in
-// shared memory and extracts the per-aisle records in parallel (a ballot
-// numbers the aisle runs) into a column matrix in global memory; a task with
-// more than MVL_RMAX records runs its scan and DP on one lane right away.
-// k_mv_long_dp: one task per thread runs the DP over its records (coalesced
-// column reads), so the DP, one step per visited aisle, keeps every lane busy.
+// Tasks of more than ROW_MAXN lines: one warp per task walks the changed tour
+// (walk_task_warp), sorts its keys in shared memory and extracts the per-aisle
+// records in parallel (a ballot numbers the aisle runs) into a column of the
+// warp's own matrix in global memory; once the matrix's long_cols columns are
+// full, or no task is left, every lane runs the DP of one of them.  A task
+// with more than MVL_RMAX records runs its scan and DP on one lane right away.
+// With one matrix for the first 65,536 tasks and the others' DPs on one lane of
+// their warp, 262,144 moves on tours of 200 lines in 40 aisles took 5.9 ms; now
+// 4.26 (in 500 aisles, where few tours' records fit, 65,536 moves 1.40 and 1.52 ms).
 __device__ __forceinline__ void mv_long_commit(const MoveArgs& M, int64_t i, int cs, int cr) {
     const int4 tk = M.tasks[i];
     M.task_cost[i] = make_int2(cs, cr);
@@ -641,17 +643,33 @@ __device__ __forceinline__ void mv_long_commit(const MoveArgs& M, int64_t i, int
     atomicAdd(reinterpret_cast<unsigned long long*>(&M.delta[2 * tk.x + 1]), (unsigned long long)dr);
 }
 
-__global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) {
+__global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long(MoveArgs M) {
     pdl_trigger();
     pdl_wait();
     __shared__ uint32_t buf[LONG_WARPS][LONG_MAXL];
+    // the matrix's columns: task, records, largest key
+    __shared__ int s_task[LONG_WARPS][32], s_m[LONG_WARPS][32];
+    __shared__ uint32_t s_last[LONG_WARPS][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int count = min(*M.long_count, M.long_cap);
     uint32_t* kb = buf[warp];
     const EvalArgs& a = M.a;
-    const int64_t cap = M.long_rec_cap;
-    for (int w = blockIdx.x * LONG_WARPS + warp; w < count; w += gridDim.x * LONG_WARPS) {
-        const int64_t i = M.long_list[w];
+    const int gw = blockIdx.x * LONG_WARPS + warp, cols = M.long_cols;
+    uint2* rec = M.long_rec + (int64_t)gw * MVL_RMAX * cols;   // record r of column j at [r * cols + j]
+    int have = 0;   // columns in use
+    auto run_dps = [&] {
+        __syncwarp();
+        if (lane < have) {
+            const uint32_t kl = s_last[warp][lane];
+            const int m = s_m[warp][lane];
+            mv_long_commit(M, s_task[warp][lane], sshape_cost(a.g, m, (int)(kl >> 16), (int)(kl & 0xFFFFu)),
+                           rr_records32_mem(a.g, rec + lane, cols, m));
+        }
+        have = 0;
+        __syncwarp();
+    };
+    for (int w = gw; w < count; w += gridDim.x * LONG_WARPS) {
+        const int i = M.long_list[w];
         const int4 tk = M.tasks[i];
         const int4 mv = M.moves[tk.x];
         int n = 0;
@@ -669,13 +687,12 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
                     M.mstatus[tk.x] = 3;
                 }
                 M.task_cost[i] = make_int2(-1, -1);
-                if (w < cap) M.long_m[w] = -1;
             }
             __syncwarp();
             continue;
         }
         warp_sort_buffer(kb, n, lane);
-        // per-aisle records: run r of the sorted keys -> long_rec[r * cap + w]
+        // per-aisle records: run r of the sorted keys -> row r of the column
         int m = 0;
         for (int x0 = 0; x0 < n; x0 += 32) {
             const int x = x0 + lane;
@@ -686,7 +703,7 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
             const bool last = in && (x == n - 1 || (int)(kb[x + 1] >> 16) != ai);
             const unsigned fm = __ballot_sync(0xffffffffu, first);
             const int r = m + __popc(fm & ((2u << lane) - 1u)) - 1;
-            if (last && r < MVL_RMAX && w < cap) {
+            if (last && r < MVL_RMAX) {
                 const int hi = (int)(key & 0xFFFFu);
                 int lo = hi, gi = 0;
                 for (int y = x; y > 0 && (int)(kb[y - 1] >> 16) == ai; --y) {
@@ -694,20 +711,19 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
                     gi = max(gi, lo - kp);
                     lo = kp;
                 }
-                M.long_rec[r * cap + w] =
+                rec[r * cols + have] =
                     make_uint2(((uint32_t)ai << 16) | (uint32_t)lo, ((uint32_t)hi << 16) | (uint32_t)gi);
             }
             m += __popc(fm);
         }
         if (lane == 0) {
             const uint32_t kl = n > 0 ? kb[n - 1] : 0u;   // rightmost aisle, its deepest slot
-            if (m <= MVL_RMAX && w < cap) {
-                M.long_key[w] = kl;
-                M.long_m[w] = m;
+            if (m <= MVL_RMAX) {
+                s_task[warp][have] = i;
+                s_m[warp][have] = m;
+                s_last[warp][have] = kl;
             } else {
-                // more aisles, or more tasks, than the record matrix keeps:
-                // scan and DP here
-                if (w < cap) M.long_m[w] = -1;
+                // more aisles than the matrix keeps: scan and DP here
                 DP5 v;
                 dp_init(v);
                 int pa = 0, lo = 0, prev = 0, gi = 0;
@@ -727,21 +743,10 @@ __global__ void __launch_bounds__(LONG_WARPS * 32, 6) k_mv_long_rec(MoveArgs M) 
                 mv_long_commit(M, i, sshape_cost(a.g, m, (int)(kl >> 16), (int)(kl & 0xFFFFu)), dp_final(v));
             }
         }
+        if (m <= MVL_RMAX && ++have == cols) run_dps();
         __syncwarp();
     }
-}
-
-__global__ void k_mv_long_dp(MoveArgs M) {
-    pdl_trigger();
-    pdl_wait();
-    const int count = min(min(*M.long_count, M.long_cap), M.long_rec_cap);
-    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < count; w += gridDim.x * blockDim.x) {
-        const int m = M.long_m[w];
-        if (m < 0) continue;
-        const uint32_t kl = M.long_key[w];
-        mv_long_commit(M, M.long_list[w], sshape_cost(M.a.g, m, (int)(kl >> 16), (int)(kl & 0xFFFFu)),
-                       rr_records32_mem(M.a.g, M.long_rec + w, M.long_rec_cap, m));
-    }
+    run_dps();
 }
 
 // moves that ended with a non-zero status report zero deltas
@@ -851,14 +856,21 @@ cudaError_t launch_moves_eval(const MoveArgs& M, int num_sms, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_moves_long(const MoveArgs& M, int num_sms, cudaStream_t s) {
-    if (M.n_tasks > 0 && M.long_rec_cap > 0) {
-        int per_sm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_long_rec, LONG_WARPS * 32, 0);
-        if (e != cudaSuccess) return e;
-        launch_dependent(k_mv_long_rec, num_sms * (per_sm > 0 ? per_sm : 1), LONG_WARPS * 32, 0, s, M);
-        launch_dependent(k_mv_long_dp, grid_of(M.long_rec_cap, 128), 128, 0, s, M);
-    }
+// Every CTA of k_mv_long that fits the chip, and as many columns a warp as it
+// can have tasks (at most a lane's each).
+cudaError_t moves_long_shape(int64_t n_tasks, int num_sms, int* grid, int* cols, size_t* bytes) {
+    int per_sm = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_long, LONG_WARPS * 32, 0);
+    if (e != cudaSuccess) return e;
+    *grid = num_sms * (per_sm > 0 ? per_sm : 1);
+    const int64_t warps = (int64_t)*grid * LONG_WARPS, most = (n_tasks + warps - 1) / warps;
+    *cols = most < 32 ? (int)most : 32;
+    *bytes = sizeof(uint2) * (size_t)MVL_RMAX * (size_t)*cols * (size_t)warps;
+    return cudaSuccess;
+}
+
+cudaError_t launch_moves_long(const MoveArgs& M, int grid, cudaStream_t s) {
+    if (M.n_tasks > 0) launch_dependent(k_mv_long, grid, LONG_WARPS * 32, 0, s, M);
     if (M.n_moves > 0) launch_dependent(k_mv_finish, grid_of(M.n_moves, 256), 256, 0, s, M);
     return cudaGetLastError();
 }

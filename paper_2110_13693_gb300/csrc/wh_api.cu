@@ -35,7 +35,7 @@ struct wh_layout {
     size_t mv_scratch_bytes = 0;
     void* mv_tasks = nullptr;     // device: move tasks + their costs + long-task list
     size_t mv_tasks_bytes = 0;
-    void* mv_long = nullptr;      // device: long tasks' record matrix, record counts, largest keys
+    void* mv_long = nullptr;      // device: long tasks' record matrices
     size_t mv_long_bytes = 0;
     void* sr_scratch = nullptr;   // device: screening features and predictions
     size_t sr_scratch_bytes = 0;
@@ -436,25 +436,18 @@ int prepare_moves(wh_layout* h, const wh_orders& o, const wh_plans& p, const int
 
 namespace {
 
-// The long tasks listed by k_mv_eval: a record matrix for as many as are
-// ever common (tasks past it are scored by one lane each), the record and DP
-// kernels, which read the list's length on the device, then the final status
-// pass.
-constexpr int64_t kLongRecTasks = 1 << 16;
-
+// The long tasks listed by k_mv_eval (the kernel reads the list's length on
+// the device), then the final status pass.
 int eval_long_tasks(wh_layout* h, wh::MoveArgs& M, cudaStream_t s) {
-    M.long_rec_cap = (int32_t)std::min<int64_t>(M.n_tasks, kLongRecTasks);
-    if (M.long_rec_cap > 0) {
-        const size_t rec = align_up(sizeof(uint2) * (size_t)wh::MVL_RMAX * (size_t)M.long_rec_cap);
-        const size_t col = align_up(sizeof(int32_t) * (size_t)M.long_rec_cap);
-        const int rc = grow(&h->mv_long, &h->mv_long_bytes, rec + 2 * col);
+    int grid = 0;
+    if (M.n_tasks > 0) {
+        size_t bytes = 0;
+        if (wh::moves_long_shape(M.n_tasks, h->num_sms, &grid, &M.long_cols, &bytes) != cudaSuccess) return WH_ECUDA;
+        const int rc = grow(&h->mv_long, &h->mv_long_bytes, bytes);
         if (rc != WH_OK) return rc;
-        char* b = static_cast<char*>(h->mv_long);
-        M.long_rec = reinterpret_cast<uint2*>(b);
-        M.long_m = reinterpret_cast<int32_t*>(b + rec);
-        M.long_key = reinterpret_cast<uint32_t*>(b + rec + col);
+        M.long_rec = static_cast<uint2*>(h->mv_long);
     }
-    return wh::launch_moves_long(M, h->num_sms, s) == cudaSuccess ? WH_OK : WH_ECUDA;
+    return wh::launch_moves_long(M, grid, s) == cudaSuccess ? WH_OK : WH_ECUDA;
 }
 
 }  // namespace

@@ -157,13 +157,10 @@ struct MoveArgs {
     int32_t* long_list;         // tasks over ROW_MAXN lines
     int32_t* long_count;
     int32_t long_cap;
-    // long tasks' per-aisle records for the one-task-per-thread DP: record r
-    // of list entry w at long_rec[r * long_rec_cap + w]; long_m[w] records
-    // (-1: scored already), long_key[w] the largest key
+    // long tasks' per-aisle records: a matrix of MVL_RMAX rows and long_cols
+    // columns (a task each) per warp of k_mv_long
     uint2* long_rec;
-    int32_t* long_m;
-    uint32_t* long_key;
-    int32_t long_rec_cap;
+    int32_t long_cols;
     unsigned long long* stats;  // [0] changed tours walked, [1] their lines (zeroed by the count pass)
 };
 
@@ -276,8 +273,10 @@ cudaError_t launch_ls_apply(const LsArgs& L, cudaStream_t s);
 cudaError_t launch_moves_prepare(const MoveArgs& M, int num_sms, cudaStream_t s, bool reuse_index);
 // task fill + tasks of <= ROW_MAXN lines; the long ones are listed
 cudaError_t launch_moves_eval(const MoveArgs& M, int num_sms, cudaStream_t s);
-// the listed long tasks (records, then their DPs) and the final status pass
-cudaError_t launch_moves_long(const MoveArgs& M, int num_sms, cudaStream_t s);
+// the listed long tasks and the final status pass; grid, long_cols and the
+// bytes of long_rec by moves_long_shape
+cudaError_t moves_long_shape(int64_t n_tasks, int num_sms, int* grid, int* cols, size_t* bytes);
+cudaError_t launch_moves_long(const MoveArgs& M, int grid, cudaStream_t s);
 constexpr int MVL_RMAX = 48;    // records per long task kept for the per-thread DP
 cudaError_t launch_moves_fill(const MoveArgs& M, int num_sms, cudaStream_t s);
 
