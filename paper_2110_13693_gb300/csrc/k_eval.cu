@@ -495,8 +495,8 @@ __device__ __forceinline__ void prep_instance(const EvalArgs& a, uint32_t mask, 
         for (int o = i0; o < a.n_orders; o += stride) a.order_pack[o] = pack_aggregate(order_aggregate(a, o));
     if (a.line_ord) {
         for (int o = i0; o < a.n_orders; o += stride) {
-            // malformed offsets and orders of 255 lines or more: k_eval_plan
-            // does not read the table then
+            // malformed offsets: k_eval_plan does not read the table then; of
+            // an order of more than ROW_MAXN lines it uses no entry
             const int lb = a.order_off[o], le = a.order_off[o + 1];
             if (lb >= 0 && le <= a.n_lines)
                 for (int l = lb; l < le; ++l) a.line_ord[l] = ((uint32_t)o << 8) | ((uint32_t)(l - lb) & 0xFFu);

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
     __shared__ uint16_t s_list[LIST];      // the round's tours by falling line count
     __shared__ uint16_t s_base[LIST];      // their rows, by tour
     __shared__ uint8_t s_n[LIST];          // their line counts, by tour
-    __shared__ int s_total, s_unit, s_rows, s_dup;
+    __shared__ int s_total, s_unit, s_rows;
     __shared__ bool s_untidy;
     const int tid = threadIdx.x, lane = tid & 31;
     uint32_t* s_dst32 = rows + a.n_lines;     // first place of an order's lines, 16 bits each (0xFFFF: none)
@@ -85,13 +85,17 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
     // (no early trigger: the long-tour kernel's blocks would take the shared
     // memory that is this one's L1)
     pdl_wait();
-    // line counts; an order book with malformed offsets or an order of 255
-    // lines or more has no line -> order table to go by
+    // line counts, up to 255 (an order of more than PL_MAXN lines makes its
+    // tour a long one); an order book with malformed offsets has no line ->
+    // order table to go by: every tour goes to the long-tour pass
+    // (2,000 plans of 4,000 orders: 207 us also with an order of 300 lines in
+    // the book, 304 with it in a tour of every plan, 222 with an order twice in
+    // every plan; 640, 953 and 656 with all tours handed over for it)
     bool odd = false;
     for (int o = tid; o < a.n_orders; o += T) {
         const int lb = a.order_off[o], le = a.order_off[o + 1];
-        const bool ok = lb >= 0 && le >= lb && le <= a.n_lines && le - lb < 255;
-        s_cnt[o] = ok ? (uint8_t)(le - lb) : 0;
+        const bool ok = lb >= 0 && le >= lb && le <= a.n_lines;
+        s_cnt[o] = ok ? (uint8_t)min(le - lb, 255) : 0;
         odd |= !ok;
     }
     if (tid == 0) s_untidy = (__ldcg(a.status) & WH_STATUS_BAD_OFFSET) != 0;
@@ -116,10 +120,10 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
             for (int i = tid; i <= PL_MAXN; i += T) s_bin[i] = 0;
             for (int i = tid; i < n_dst; i += T) s_dst32[i] = 0xFFFFFFFFu;
             for (int i = tid; i < n_seen; i += T) s_seen[i] = 0u;
-            if (tid == 0) s_unit = s_rows = s_dup = 0;
+            if (tid == 0) s_unit = s_rows = 0;
             __syncthreads();
             // ---- count
-            int at[PL_U];   // place in the tour's bin, -1: not scored here
+            int at[PL_U];   // line count << 16 | place in its bin, -1: not scored here
 #pragma unroll
             for (int u = 0; u < PL_U; ++u) {
                 const int i = tid + u * T;
@@ -132,39 +136,33 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
                     if (a.tour_rr) a.tour_rr[tb + i] = -1;
                     continue;
                 }
-                s_n[i] = (uint8_t)min(n, 255);
-                at[u] = 0;
-                if (odd || n > PL_MAXN) continue;
-                int pos = atomicAdd(&s_rows, n);
-                if (pos + n > a.n_lines) {   // more lines than the book has: an order is taken twice
-                    s_dup = 1;
-                    continue;
-                }
-                s_base[i] = (uint16_t)pos;
-                at[u] = atomicAdd(&s_bin[n], 1);
-                for (int q = q0; q < q1; q += 4) {
-                    int o[4];
+                // the long-tour pass takes tours of too many lines, tours that
+                // want an order which another place has already, and the tours
+                // that the rows have no room for then
+                const int base = !odd && n <= PL_MAXN ? atomicAdd(&s_rows, n) : a.n_lines + 1;
+                if (base + n <= a.n_lines) {
+                    s_n[i] = (uint8_t)n;
+                    s_base[i] = (uint16_t)base;
+                    at[u] = n << 16 | atomicAdd(&s_bin[n], 1);
+                    int pos = base;
+                    bool taken = false;
+                    for (int q = q0; q < q1; q += 4) {
+                        int o[4];
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) o[v] = q + v < q1 ? __ldg(a.order_seq + q + v) : -1;
+                        for (int v = 0; v < 4; ++v) o[v] = q + v < q1 ? __ldg(a.order_seq + q + v) : -1;
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        if (o[v] < 0) continue;
-                        const uint32_t bit = 1u << (o[v] & 31);
-                        if (atomicOr(&s_seen[o[v] >> 5], bit) & bit) s_dup = 1;
-                        s_dst[o[v]] = (uint16_t)pos;
-                        pos += s_cnt[o[v]];
+                        for (int v = 0; v < 4; ++v) {
+                            if (o[v] < 0) continue;
+                            const int cnt = s_cnt[o[v]];
+                            const uint32_t bit = cnt > 0 ? 1u << (o[v] & 31) : 0u;
+                            if (atomicOr(&s_seen[o[v] >> 5], bit) & bit) taken = true;
+                            else s_dst[o[v]] = (uint16_t)pos;
+                            pos += cnt;
+                        }
                     }
+                    if (!taken) continue;
+                    s_n[i] = 0;   // it keeps its place in the list, as a tour of no lines
                 }
-            }
-            __syncthreads();
-            const bool all_long = odd || s_dup;
-            // tours that the long-tour pass takes: too many lines, or (all of
-            // them) an order book or a plan whose lines have no single place
-#pragma unroll
-            for (int u = 0; u < PL_U; ++u) {
-                const int i = tid + u * T;
-                if (at[u] < 0 || !(all_long || s_n[i] > PL_MAXN)) continue;
-                at[u] = -1;
                 const int slot = atomicAdd(a.long_count, 1);
                 if (slot < a.long_cap) {
                     a.long_list[3 * slot] = 0;
@@ -176,10 +174,8 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
                     if (a.tour_rr) a.tour_rr[tb + i] = -1;
                 }
             }
-            if (all_long) {
-                __syncthreads();   // s_dup is reset next
-                continue;
-            }
+            __syncthreads();
+            if (odd) continue;   // (every tour handed over)
             // the bins' first places in the list: most lines first
             if (tid < 32) {
                 constexpr int B = (PL_MAXN + 32) / 32;
@@ -231,7 +227,7 @@ __global__ void __launch_bounds__(PL_THREADS, CTAS) k_eval_plan(EvalArgs a) {
             __syncthreads();
 #pragma unroll
             for (int u = 0; u < PL_U; ++u)
-                if (at[u] >= 0) s_list[s_bin[s_n[tid + u * T]] + at[u]] = (uint16_t)(tid + u * T);
+                if (at[u] >= 0) s_list[s_bin[at[u] >> 16] + (at[u] & 0xFFFF)] = (uint16_t)(tid + u * T);
             __syncthreads();
             // ---- sort: units of a warp's tours, the longest first
             const int total = s_total, c8 = s_bin[64], c4 = s_bin[32];   // tours over 64 and over 32 lines

@@ -54,3 +54,33 @@ def test_empty_tours_beside_long_ones(gpu_lib, case):
         w = np.where(hit, -1, want[k])
         assert np.array_equal(got[k], w)
         assert np.array_equal(got[2 + k], np.bincount(plan_of, np.where(hit, 0, w)).astype(np.int64))
+
+
+@pytest.mark.parametrize("own", [True, False])
+@pytest.mark.parametrize("case", ["long_unused", "long_in_some", "empty_twice", "all_twice", "twice_in_one", "rows_full"])
+def test_tours_handed_over_one_by_one(gpu_lib, case, own):
+    """Orders of over 128 and over 255 lines, and orders taken twice: beside tours without them."""
+    lay, rng, n_sku = LAYOUTS["wide"], np.random.default_rng(8), 700
+    sizes = rng.integers(0, 9, 1500)
+    sizes[[5, 6]] = 3
+    if case.startswith("long"):
+        sizes[[40, 41, 42, 43, 44]] = 128, 129, 254, 255, 900
+    if case == "empty_twice":
+        sizes[5] = 0
+    orders = [rng.integers(0, n_sku, k).tolist() for k in sizes]
+    plans = cut(rng, len(orders), 160, 9, empty=(4,))      # (enough plans for a shared slotting to come here)
+    for k, plan in enumerate(plans):
+        if case == "long_unused":
+            plan[:] = [[o for o in t if o not in range(40, 45)] for t in plan]
+        elif case in ("empty_twice", "twice_in_one"):
+            a, b = (3, 3) if case == "twice_in_one" else (k % 50, 60)
+            plan[a], plan[b] = plan[a] + [5], plan[b] + [5]
+        elif case == "all_twice":
+            plan[:] = plan + cut(rng, len(orders), 1, 7)[0]
+        elif case == "rows_full":                          # the same orders over and over: more lines than the book has
+            plan[:] = plan + [t[::-1] for t in plan[:120]] * 2
+    inst = make_instance(lay, orders, rng.permutation(lay.n_loc)[:n_sku], plans, n_sku)
+    maps = own_maps(lay, rng, len(plans), n_sku) if own else None
+    got = gpu_eval(gpu_lib, inst, slot_map=maps, stride=n_sku if own else 0, prefill=-9)
+    assert got[4] == 0
+    assert_exact(got, oracle.eval_plans(inst, **(dict(slot_map=maps, slot_map_stride=n_sku) if own else {})))
