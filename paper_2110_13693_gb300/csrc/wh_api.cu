@@ -78,8 +78,8 @@ struct wh_batch {
 };
 
 namespace {
-enum KernelId { K_PREP = 0, K_EVAL_SHORT = 1, K_EVAL_LONG = 2, K_EVAL_SSHAPE = 3, K_COUNT = 4 };
-const char* const kKernelNames[K_COUNT] = {"k_prep", "k_eval_short", "k_eval_long", "k_eval_sshape"};
+enum KernelId { K_PREP = 0, K_EVAL_SHORT = 1, K_EVAL_LONG = 2, K_EVAL_SSHAPE = 3, K_EVAL_PLAN = 4, K_COUNT = 5 };
+const char* const kKernelNames[K_COUNT] = {"k_prep", "k_eval_short", "k_eval_long", "k_eval_sshape", "k_eval_plan"};
 
 // Brackets one launch with events when timing is on.
 class LaunchTimer {
@@ -337,7 +337,7 @@ extern "C" int wh_eval_plans(wh_layout* h, const wh_orders* orders, const wh_pla
         if (!lt.ok() || wh::launch_prep(a, s) != cudaSuccess) return WH_ECUDA;
     }
     {
-        LaunchTimer lt(h->timing, wh::sshape_kernel_applies(a) ? K_EVAL_SSHAPE : K_EVAL_SHORT, s);
+        LaunchTimer lt(h->timing, per_plan ? K_EVAL_PLAN : wh::sshape_kernel_applies(a) ? K_EVAL_SSHAPE : K_EVAL_SHORT, s);
         if (!lt.ok()) return WH_ECUDA;
         const cudaError_t e = per_plan ? wh::launch_eval_plan(a, h->num_sms, s)
                                        : wh::launch_eval_short(a, t, h->num_sms, s, nullptr);
