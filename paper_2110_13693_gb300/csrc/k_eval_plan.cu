@@ -279,6 +279,33 @@ size_t plan_smem_bytes(const EvalArgs& a) {
            (((size_t)a.n_orders + 15) & ~(size_t)15);
 }
 
+// Four CTAs an SM and lists of 512 tours instead of three and 1,024 (launch_eval_plan).
+bool four_ctas(const EvalArgs& a) {
+    return plan_smem_bytes(a) <= (a.slot_stride == 0 ? 53 : 40) * 1024 && a.n_tours <= 448ll * a.n_plans;
+}
+
+// k_eval_short walks what the plans hold; here every plan has the whole order
+// book translated, again for every round of its tours, and a thread for every
+// tour.  Microseconds of either beyond what both take, as they were measured
+// over 792 shapes (books of 600 to 4,000 orders, plans that hold 32 orders to
+// all of them in tours of 1 to 24, 16 to 2,000 plans; own slottings of 200,000
+// and of 8,000 locations and shared ones): k_eval_short's chain of loads per
+// line or its lines' throughput, this kernel's latency for a book and its
+// tours or its throughput.
+bool short_is_faster(const EvalArgs& a) {
+    const bool own = a.slot_stride != 0;
+    const double plans = a.n_plans, book = a.n_lines, tours = a.n_tours / plans;
+    const double held = a.n_orders > 0 ? book * ((double)a.n_seq / a.n_orders) / plans : 0.0, lines = held / tours;
+    const double rounds = 1 + (int)(tours / (four_ctas(a) ? 512 : 1024));
+    const double chain = (!own ? 0.6 : key16_ok(a.g) ? 1.8 : 1.0) * lines;
+    const double walk = (own ? 25e-6 : 14.5e-6) * plans * held;
+    const double latency = (own ? 0.7e-3 : 0.5e-3) * rounds * book + 18e-3 * tours + 0.18 * lines;
+    const double work = own ? rounds * (13e-3 + 5e-6 * book) + 2.5e-6 * held + 23e-6 * tours
+                            : rounds * (13e-3 + 0.6e-6 * book) + 5e-6 * held + 30e-6 * tours;
+    const double both = 16.0;
+    return both + (latency > plans * work ? latency : plans * work) > 1.1 * (both + (chain > walk ? chain : walk));
+}
+
 }  // namespace
 
 // Measured against k_eval_short + k_eval_long (us a call, GB300; orders x
@@ -293,17 +320,29 @@ size_t plan_smem_bytes(const EvalArgs& a) {
 //                    400 x 17 x 59: 152 plans 37 -> 19, 2,000 plans 50 -> 72
 //                    3,000 x 375 x 20: 64 plans 25 -> 29, 152 plans 29 -> 27,
 //                    2,000 plans 206 -> 99
+//   own, 4,000 orders in the book, 500 aisles
+//                    all held, a tour each: 16 plans 18 -> 105, 600 plans 204 -> 271
+//                    128 held, a tour each: 2,000 plans 42 -> 124
+//                    512 held, 8 a tour: 16 plans 38 -> 26, 2,000 plans 80 -> 134
+//                    1,000 held, 24 a tour: 16 plans 67 -> 33, 600 plans 86 -> 76
 // So: many plans of few tours (a CTA's threads idle, and one tour per thread
-// fills the chip anyway) and few plans of short tours under a shared slotting
-// (k_eval_short has no latency of gathers or of a long-tour pass there) stay.
+// fills the chip anyway), few plans of short tours under a shared slotting
+// (k_eval_short has no latency of gathers or of a long-tour pass there) and
+// short tours or small parts of a large book where that tells (short_is_faster)
+// stay.  With the last of them left out, the 792 shapes take on average 18 %
+// more than the faster of the two, with it 2 %.
 // Three CTAs an SM take order books of up to 67 KB; a shared slotting with
 // 16-bit keys is k_eval_short's best case (half the sort, one gather).
 bool eval_plan_applies(const EvalArgs& a, int num_sms) {
     if (sshape_kernel_applies(a) || a.n_tours == 0 || a.n_lines > 0xFFFE || plan_smem_bytes(a) > 67 * 1024) return false;
     if (a.n_plans > 4 * num_sms && a.n_tours / a.n_plans < 64) return false;
-    if (a.slot_stride != 0) return true;
-    if (key16_ok(a.g)) return false;
-    return a.n_plans >= num_sms || (double)a.n_lines * (double)a.n_seq > 32.0 * (double)a.n_orders * (double)a.n_tours;
+    if (a.slot_stride == 0) {
+        if (key16_ok(a.g)) return false;
+        if (a.n_plans < num_sms &&
+            (double)a.n_lines * (double)a.n_seq <= 32.0 * (double)a.n_orders * (double)a.n_tours)
+            return false;
+    }
+    return !short_is_faster(a);
 }
 
 // Three CTAs an SM (60 KB an order book at paper scale; what is left of the
@@ -315,7 +354,7 @@ bool eval_plan_applies(const EvalArgs& a, int num_sms) {
 cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s) {
     const size_t smem = plan_smem_bytes(a);
     const bool shared = a.slot_stride == 0;
-    const bool four = smem <= (shared ? 53 : 40) * 1024 && a.n_tours <= 448ll * a.n_plans;
+    const bool four = four_ctas(a);
     auto kern = shared ? (four ? k_eval_plan<true, 512, 4> : k_eval_plan<true, 1024, 3>)
                        : (four ? k_eval_plan<false, 512, 4> : k_eval_plan<false, 1024, 3>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -19,8 +19,8 @@ pytestmark = pytest.mark.gpu
 def test_malformed_plan_offsets(gpu_lib, case, own, n_plans):
     import paper_2110_13693_gb300 as wh
     lay, rng, n_sku = wh_gen.Layout(260, 4), np.random.default_rng(n_plans), 300
-    orders = [rng.integers(0, n_sku, k).tolist() for k in rng.integers(1, 5, 192)]
-    inst = make_instance(lay, orders, rng.permutation(lay.n_loc)[:n_sku], cut(rng, len(orders), n_plans, 3), n_sku)
+    orders = [rng.integers(0, n_sku, k).tolist() for k in rng.integers(1, 8, 512)]
+    inst = make_instance(lay, orders, rng.permutation(lay.n_loc)[:n_sku], cut(rng, len(orders), n_plans, 8), n_sku)
     maps = own_maps(lay, rng, n_plans, n_sku) if own else None
     off = inst.plan_tour_off.copy()
     if case == "first":
