@@ -105,10 +105,10 @@ __device__ __forceinline__ void row_costs(const Geo& g, const DPConst& c, const 
 // A warp takes up to 32 tours, one a lane, possibly changed by a move, as
 // many of one plan at a time as its rows of shared memory hold.  Tour by tour
 // the lanes take the tour's orders (the next tours' ids and line ranges in
-// flight) and put its lines' SKUs, the moved ones already exchanged, into the
-// tour's row; then the slot-map gathers of all rows run flat, eight a lane in
-// flight; then the rows are sorted (sort_rows).  No dependent gather per line
-// and few registers.
+// flight), or every lane takes its own tour's where they are few, and put its
+// lines' SKUs, the moved ones already exchanged, into the tour's row; then the
+// slot-map gathers of all rows run flat, eight a lane in flight; then the rows
+// are sorted (sort_rows).  No dependent gather per line and few registers.
 constexpr int ROW_WARPS = 4;                // warps of a CTA
 constexpr int ROW_THREADS = ROW_WARPS * 32;
 constexpr int ROW_WORDS = 2048;             // keys of a warp's rows: 32 tours of 64 lines
@@ -155,6 +155,51 @@ cudaError_t rows_per_sm(K kern, int* per_sm) {
     return e;
 }
 
+// The tour of one lane into its row, order by order (four orders' ids and line
+// ranges, then four lines' SKUs, in flight), the move applied.
+__device__ __forceinline__ void walk_row_lane(const EvalArgs& a, const RowTour& w, uint32_t* row, int& n, bool& primary) {
+    const bool swap = w.mv.x >= 2;
+    const int rem = !swap && w.tk.w >= 0 ? w.tk.w : -1, q_end = w.add >= 0 ? w.q1 + 1 : w.q1;
+    int hit_min = 0x7fffffff;
+    bool own_has_s1 = false;
+    uint32_t* at = row;
+    for (int q = w.q0; q < q_end; q += 4) {
+        int o[4], lb[4], le[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) o[u] = q + u < w.q1 ? a.order_seq[q + u] : q + u < q_end ? w.add : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            lb[u] = le[u] = 0;
+            if (o[u] >= 0 && !(q + u < w.q1 && o[u] == rem)) {
+                lb[u] = a.order_off[o[u]];
+                le[u] = a.order_off[o[u] + 1];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            for (int l = lb[u]; l < le[u]; l += 4) {
+                uint32_t sk[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) sk[v] = l + v < le[u] ? (uint32_t)a.line_sku[l + v] : SKU_BAD;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    if (l + v >= le[u]) continue;
+                    uint32_t k = sk[v] < (uint32_t)a.n_sku ? sk[v] : SKU_BAD;
+                    const bool s1 = k == (uint32_t)w.mv.y;
+                    if (swap && (s1 || (w.mv.x == 2 && k == (uint32_t)w.mv.z))) {
+                        hit_min = min(hit_min, o[u]);
+                        own_has_s1 |= s1 && o[u] == w.tk.z;
+                        k = w.mv.x == 3 ? SKU_AT | (uint32_t)w.mv.z : (uint32_t)(s1 ? w.mv.z : w.mv.y);
+                    }
+                    *at++ = k;
+                }
+            }
+        }
+    }
+    n = (int)(at - row);
+    primary = !swap || (hit_min == w.tk.z && (w.tk.w == -2 || !own_has_s1));
+}
+
 // Runs the lanes of `todo`.  For every batch done(mine, primary, base, n, bad)
 // is called by the whole warp: whether this lane's task is in the batch,
 // whether it is the counted one of its tour (only those rows are sorted), its
@@ -180,134 +225,142 @@ __device__ __forceinline__ void run_rows(const EvalArgs& a, uint32_t* rows, RowL
         const int32_t* map = a.slot_map + (int64_t)plan * a.slot_stride;
         bool primary = true;
         int n = 0;
-        // ids two tasks ahead, line ranges one task ahead
-        int j = __ffs(take) - 1, j2 = j;
-        unsigned left = take & (take - 1);
-        auto first_ids = [&](int k) {
-            const int b0 = __shfl_sync(0xffffffffu, w.q0, k), b1 = __shfl_sync(0xffffffffu, w.q1, k);
-            return b0 + lane < b1 ? a.order_seq[b0 + lane] : -1;
-        };
-        int o_cur = first_ids(j), o_nxt = -1;
-        int lb_cur = 0, le_cur = 0;
-        if (o_cur >= 0) {
-            lb_cur = a.order_off[o_cur];
-            le_cur = a.order_off[o_cur + 1];
-        }
-        if (left) {
-            j2 = __ffs(left) - 1;
-            o_nxt = first_ids(j2);
-        }
-        for (;;) {
-            const int b0 = __shfl_sync(0xffffffffu, w.q0, j), b1 = __shfl_sync(0xffffffffu, w.q1, j);
-            const int jadd = __shfl_sync(0xffffffffu, w.add, j), jbase = __shfl_sync(0xffffffffu, base, j);
-            const int type = __shfl_sync(0xffffffffu, w.mv.x, j);
-            const int mb = __shfl_sync(0xffffffffu, w.mv.y, j), mc = __shfl_sync(0xffffffffu, w.mv.z, j);
-            const int tz = __shfl_sync(0xffffffffu, w.tk.z, j), tw = __shfl_sync(0xffffffffu, w.tk.w, j);
-            const int jj = j;
-            const bool more = left != 0;
-            int o0 = o_cur, lb0 = lb_cur, le0 = le_cur;   // this lane's order of the first 32
-            j = j2;
-            o_cur = o_nxt;
-            lb_cur = le_cur = 0;
-            if (more) {
-                if (o_cur >= 0) {
-                    lb_cur = a.order_off[o_cur];
-                    le_cur = a.order_off[o_cur + 1];
-                }
-                left &= left - 1;
-                if (left) {
-                    j2 = __ffs(left) - 1;
-                    o_nxt = first_ids(j2);
-                }
+        const int orders = mine ? w.q1 - w.q0 + (w.add >= 0 ? 1 : 0) : 0;
+        if (3 * (int)__reduce_max_sync(0xffffffffu, (unsigned)orders) <= 2 * __popc(take)) {
+            // every lane its own: 131,072 moves on tours of one order 330 us
+            // tour by tour, 211 so, and with a very popular SKU 580 and 301
+            // (of 16 orders 357 and 333; of 24 it takes as long or longer)
+            if (mine) walk_row_lane(a, w, rows + base, n, primary);
+        } else {
+            // ids two tasks ahead, line ranges one task ahead
+            int j = __ffs(take) - 1, j2 = j;
+            unsigned left = take & (take - 1);
+            auto first_ids = [&](int k) {
+                const int b0 = __shfl_sync(0xffffffffu, w.q0, k), b1 = __shfl_sync(0xffffffffu, w.q1, k);
+                return b0 + lane < b1 ? a.order_seq[b0 + lane] : -1;
+            };
+            int o_cur = first_ids(j), o_nxt = -1;
+            int lb_cur = 0, le_cur = 0;
+            if (o_cur >= 0) {
+                lb_cur = a.order_off[o_cur];
+                le_cur = a.order_off[o_cur + 1];
             }
-            const bool swap = type >= 2;
-            const int rem = !swap && tw >= 0 ? tw : -1;
-            const int b_end = jadd >= 0 ? b1 + 1 : b1;
-            if (b0 + lane < b1) {
-                if (o0 == rem) lb0 = le0 = 0;
-            } else if (b0 + lane < b_end) {   // the added order comes last
-                o0 = jadd;
-                lb0 = a.order_off[o0];
-                le0 = a.order_off[o0 + 1];
+            if (left) {
+                j2 = __ffs(left) - 1;
+                o_nxt = first_ids(j2);
             }
-            uint32_t* row = rows + jbase;
-            // the lines' indices at their places (lanes over orders;
-            // ids and line counts were checked with the tour's count)
-            int cnt_all = 0;
-            for (int qb = b0; qb < b_end; qb += 32) {
-                int lb = lb0, le = le0;
-                if (qb > b0) {
-                    const int q = qb + lane;
-                    lb = le = 0;
-                    if (q < b_end) {
-                        const int o = q < b1 ? a.order_seq[q] : jadd;
-                        if (!(q < b1 && o == rem)) {
-                            lb = a.order_off[o];
-                            le = a.order_off[o + 1];
-                        }
+            for (;;) {
+                const int b0 = __shfl_sync(0xffffffffu, w.q0, j), b1 = __shfl_sync(0xffffffffu, w.q1, j);
+                const int jadd = __shfl_sync(0xffffffffu, w.add, j), jbase = __shfl_sync(0xffffffffu, base, j);
+                const int type = __shfl_sync(0xffffffffu, w.mv.x, j);
+                const int mb = __shfl_sync(0xffffffffu, w.mv.y, j), mc = __shfl_sync(0xffffffffu, w.mv.z, j);
+                const int tz = __shfl_sync(0xffffffffu, w.tk.z, j), tw = __shfl_sync(0xffffffffu, w.tk.w, j);
+                const int jj = j;
+                const bool more = left != 0;
+                int o0 = o_cur, lb0 = lb_cur, le0 = le_cur;   // this lane's order of the first 32
+                j = j2;
+                o_cur = o_nxt;
+                lb_cur = le_cur = 0;
+                if (more) {
+                    if (o_cur >= 0) {
+                        lb_cur = a.order_off[o_cur];
+                        le_cur = a.order_off[o_cur + 1];
+                    }
+                    left &= left - 1;
+                    if (left) {
+                        j2 = __ffs(left) - 1;
+                        o_nxt = first_ids(j2);
                     }
                 }
-                const int cnt = le - lb;
-                const int inc = warp_inclusive_scan(cnt);
-                uint32_t* at = row + cnt_all + inc - cnt;
-                for (int l = lb; l < le; ++l) *at++ = (uint32_t)l;
-                cnt_all += __shfl_sync(0xffffffffu, inc, 31);
-            }
-            __syncwarp();
-            // their SKUs, the move applied: an exchanged SKU takes the
-            // other's place, a relocated one its new location
-            int hit_min = 0x7fffffff;
-            bool own_has_s1 = false;
-            for (int x0 = 0; x0 < cnt_all; x0 += 64) {
-                int l[2];
-                uint32_t sk[2];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int x = x0 + 32 * u + lane;
-                    l[u] = x < cnt_all ? (int)row[x] : -1;
-                    sk[u] = l[u] >= 0 ? (uint32_t)a.line_sku[l[u]] : SKU_BAD;
+                const bool swap = type >= 2;
+                const int rem = !swap && tw >= 0 ? tw : -1;
+                const int b_end = jadd >= 0 ? b1 + 1 : b1;
+                if (b0 + lane < b1) {
+                    if (o0 == rem) lb0 = le0 = 0;
+                } else if (b0 + lane < b_end) {   // the added order comes last
+                    o0 = jadd;
+                    lb0 = a.order_off[o0];
+                    le0 = a.order_off[o0 + 1];
                 }
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    uint32_t k = sk[u] < (uint32_t)a.n_sku ? sk[u] : SKU_BAD;
-                    if (swap) {
-                        const bool s1 = k == (uint32_t)mb, hit = s1 || (type == 2 && k == (uint32_t)mc);
-                        // a moved SKU's line: the order that holds it
-                        // (a SKU move keeps every order of the tour)
-                        for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1) {
-                            const int src = __ffs(hits) - 1;
-                            const int hl = __shfl_sync(0xffffffffu, l[u], src);
-                            const bool h1 = __shfl_sync(0xffffffffu, (int)s1, src) != 0;
-                            for (int qb = b0; qb < b1; qb += 32) {
-                                int o = o0, lb = lb0, le = le0;
-                                if (qb > b0) {
-                                    lb = le = 0;
-                                    if (qb + lane < b1) {
-                                        o = a.order_seq[qb + lane];
-                                        lb = a.order_off[o];
-                                        le = a.order_off[o + 1];
-                                    }
-                                }
-                                if (hl >= lb && hl < le) {
-                                    hit_min = min(hit_min, o);
-                                    own_has_s1 |= h1 && o == tz;
-                                }
+                uint32_t* row = rows + jbase;
+                // the lines' indices at their places (lanes over orders;
+                // ids and line counts were checked with the tour's count)
+                int cnt_all = 0;
+                for (int qb = b0; qb < b_end; qb += 32) {
+                    int lb = lb0, le = le0;
+                    if (qb > b0) {
+                        const int q = qb + lane;
+                        lb = le = 0;
+                        if (q < b_end) {
+                            const int o = q < b1 ? a.order_seq[q] : jadd;
+                            if (!(q < b1 && o == rem)) {
+                                lb = a.order_off[o];
+                                le = a.order_off[o + 1];
                             }
                         }
-                        if (hit) k = type == 3 ? SKU_AT | (uint32_t)mc : (uint32_t)(s1 ? mc : mb);
                     }
-                    if (l[u] >= 0) row[x0 + 32 * u + lane] = k;
+                    const int cnt = le - lb;
+                    const int inc = warp_inclusive_scan(cnt);
+                    uint32_t* at = row + cnt_all + inc - cnt;
+                    for (int l = lb; l < le; ++l) *at++ = (uint32_t)l;
+                    cnt_all += __shfl_sync(0xffffffffu, inc, 31);
                 }
+                __syncwarp();
+                // their SKUs, the move applied: an exchanged SKU takes the
+                // other's place, a relocated one its new location
+                int hit_min = 0x7fffffff;
+                bool own_has_s1 = false;
+                for (int x0 = 0; x0 < cnt_all; x0 += 64) {
+                    int l[2];
+                    uint32_t sk[2];
+    #pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int x = x0 + 32 * u + lane;
+                        l[u] = x < cnt_all ? (int)row[x] : -1;
+                        sk[u] = l[u] >= 0 ? (uint32_t)a.line_sku[l[u]] : SKU_BAD;
+                    }
+    #pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        uint32_t k = sk[u] < (uint32_t)a.n_sku ? sk[u] : SKU_BAD;
+                        if (swap) {
+                            const bool s1 = k == (uint32_t)mb, hit = s1 || (type == 2 && k == (uint32_t)mc);
+                            // a moved SKU's line: the order that holds it
+                            // (a SKU move keeps every order of the tour)
+                            for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1) {
+                                const int src = __ffs(hits) - 1;
+                                const int hl = __shfl_sync(0xffffffffu, l[u], src);
+                                const bool h1 = __shfl_sync(0xffffffffu, (int)s1, src) != 0;
+                                for (int qb = b0; qb < b1; qb += 32) {
+                                    int o = o0, lb = lb0, le = le0;
+                                    if (qb > b0) {
+                                        lb = le = 0;
+                                        if (qb + lane < b1) {
+                                            o = a.order_seq[qb + lane];
+                                            lb = a.order_off[o];
+                                            le = a.order_off[o + 1];
+                                        }
+                                    }
+                                    if (hl >= lb && hl < le) {
+                                        hit_min = min(hit_min, o);
+                                        own_has_s1 |= h1 && o == tz;
+                                    }
+                                }
+                            }
+                            if (hit) k = type == 3 ? SKU_AT | (uint32_t)mc : (uint32_t)(s1 ? mc : mb);
+                        }
+                        if (l[u] >= 0) row[x0 + 32 * u + lane] = k;
+                    }
+                }
+                if (swap) {
+                    hit_min = __reduce_min_sync(0xffffffffu, hit_min);
+                    own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
+                }
+                if (lane == jj) {
+                    n = cnt_all;
+                    primary = !swap || (hit_min == tz && (tw == -2 || !own_has_s1));
+                }
+                if (!more) break;
             }
-            if (swap) {
-                hit_min = __reduce_min_sync(0xffffffffu, hit_min);
-                own_has_s1 = __any_sync(0xffffffffu, own_has_s1);
-            }
-            if (lane == jj) {
-                n = cnt_all;
-                primary = !swap || (hit_min == tz && (tw == -2 || !own_has_s1));
-            }
-            if (!more) break;
         }
         __syncwarp();
         // keys, all rows at once (what lies between rows is translated
