@@ -1168,7 +1168,15 @@ size_t eval_batch_smem_bytes(const BatchArgs& b, const Tuning& t, bool k16) {
     return s + buffer_bytes(k16, b.max_rec, t.threads);
 }
 
-bool sshape_packs(const Geo& g, int32_t n_orders) { return g.A <= 50 && g.L <= 256 && n_orders <= SSHAPE_PACK_ORDERS; }
+// Of more than 9,600 orders an SM holds two tables (32 warps) instead of three,
+// too few to hide the start of every tour where tours are short: 12,000 orders,
+// 1,024 plans, in us with 16-byte and with packed records: tours of 1 order 132
+// and 169, of 4 48 and 54, of 8 42 and 39, of 20 48 and 36 (8,000 orders: 94
+// and 95, 36 and 36, 33 and 28, 33 and 28).
+bool sshape_packs(const EvalArgs& a) {
+    return a.g.A <= 50 && a.g.L <= 256 && a.n_orders <= SSHAPE_PACK_ORDERS &&
+           (a.n_orders <= 9600 || a.n_seq >= 8 * (int64_t)a.n_tours);
+}
 
 static cudaError_t launch_sshape(const EvalArgs& a, const Tuning& t, int num_sms, cudaStream_t s, int* grid_out) {
     if (a.order_pack) {

@@ -325,7 +325,7 @@ extern "C" int wh_eval_plans(wh_layout* h, const wh_orders* orders, const wh_pla
     if (rc != WH_OK) return rc;
     char* base = static_cast<char*>(h->scratch);
     a.line_key = shared_map && !agg && o.n_lines > 0 ? reinterpret_cast<uint32_t*>(base) : nullptr;
-    const bool pack = agg && wh::sshape_packs(h->g, o.n_orders);
+    const bool pack = agg && wh::sshape_packs(a);
     a.order_agg = agg && !pack ? reinterpret_cast<uint4*>(base + key_bytes) : nullptr;
     a.order_pack = pack ? reinterpret_cast<uint2*>(base + key_bytes) : nullptr;
     a.long_list = reinterpret_cast<int32_t*>(base + key_bytes + agg_bytes);

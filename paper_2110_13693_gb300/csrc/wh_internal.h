@@ -369,7 +369,7 @@ bool sshape_kernel_applies(const EvalArgs& a);
 // the S-shape-only kernel takes packed per-order records (k_eval_sshape_pack):
 // order books of up to 96 KB of them, two CTAs an SM
 constexpr int32_t SSHAPE_PACK_ORDERS = 12288;
-bool sshape_packs(const Geo& g, int32_t n_orders);
+bool sshape_packs(const EvalArgs& a);
 // one CTA per plan (k_eval_plan.cu) instead of one tour per thread (launch_eval_short)
 bool eval_plan_applies(const EvalArgs& a, int num_sms);
 cudaError_t launch_eval_plan(const EvalArgs& a, int num_sms, cudaStream_t s);
