@@ -583,7 +583,7 @@ def run_kmeans(wh, dev, cpu=True):
 
 def run_routes(wh, dev, cpu=True):
     """Explicit optimal pick sequences for every tour of 1,024 paper-scale
-    plans (one thread per tour: tracking DP, backtrack, Euler circuit), one
+    plans (one warp per tour: DP, arrival codes, backtrack, Euler circuit), one
     launch after a warm-up; the route lengths are checked against the
     evaluator's optimal tour lengths."""
     import torch

@@ -174,10 +174,11 @@ int wh_eval_plans(wh_layout *layout, const wh_orders *orders, const wh_plans *pl
  * range, order not in the plan, SKU move under a shared slotting, relocation
  * onto an occupied location or without loc_used, or a malformed tour); deltas are 0 unless
  * the status is 0.  Each plan must hold every order at most once.
- * All arrays are device memory.  The call synchronises `stream` twice (to
- * size its task list, then the record matrix of the tasks of more than 64
- * lines) and may allocate scratch.  Returns WH_OK, WH_EINVAL, WH_ENOMEM
- * or WH_ECUDA. */
+ * An order counts once for a SKU move, also where it asks for the SKU on
+ * several of its lines.  All arrays are device memory.  The call synchronises
+ * `stream` once (to size its task list) and may allocate scratch (with it the
+ * record matrices of the tasks of more than 128 lines, up to 45 MB).  Returns
+ * WH_OK, WH_EINVAL, WH_ENOMEM or WH_ECUDA. */
 int wh_eval_moves(wh_layout *layout, const wh_orders *orders, const wh_plans *plans, const int32_t *tour_s,
                   const int32_t *tour_rr, const int32_t *moves, int32_t n_moves, int32_t max_orders_per_tour,
                   int32_t max_lines_per_tour, int64_t *delta, int32_t *status, void *stream);
@@ -297,8 +298,8 @@ int wh_kmeans_slotting(wh_layout *layout, const wh_orders *orders, const int8_t 
  * covers exactly length[i].  A tour with more than min(max_points, 256)
  * distinct points sets WH_STATUS_TOUR_TOO_LONG; a bad tour index or offsets
  * WH_STATUS_BAD_OFFSET; bad ids WH_STATUS_BAD_ORDER / WH_STATUS_BAD_LOC.  One
- * thread per tour, about 10 KB of local memory each; meant for the tours of
- * a chosen plan, not for scoring.  Asynchronous on `stream`; allocates
+ * warp per tour, about 11 KB of shared memory each; meant for the tours of
+ * chosen plans, not for scoring.  Asynchronous on `stream`; allocates
  * nothing.  Returns WH_OK, WH_EINVAL or WH_ECUDA. */
 int wh_routes(wh_layout *layout, const wh_orders *orders, const wh_plans *plans, const int32_t *tours, int32_t n,
               int32_t max_points, int32_t *points, int32_t *n_points, int32_t *length, void *stream);

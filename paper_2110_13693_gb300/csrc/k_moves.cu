@@ -993,11 +993,11 @@ __global__ void k_ls_apply(LsArgs L) {
     }
 }
 
-// Features of every task's changed tour, one task per warp (WarpFeat): the
-// same walk as walk_task with lane j taking the tour's orders j, j + 32, ...
-// (the added order last); the SKU-swap rule that picks the counted task of
-// a tour reduces over the lanes.  Marks in task_cost which tasks count
-// (rows of non-counted tasks are written too and ignored by the selection).
+// Features of every task's changed tour, one task per warp (WarpFeat): its
+// orders by the lanes, the added one last; the SKU-swap rule that picks the
+// counted task of a tour reduces over the lanes.  Marks in task_cost which
+// tasks count (rows of non-counted tasks are written too and ignored by the
+// selection).
 constexpr int TF_THREADS = 256;
 
 // One changed tour per warp.  Its orders are taken 32 at a time (one per
