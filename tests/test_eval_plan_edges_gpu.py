@@ -68,15 +68,15 @@ def test_tours_handed_over_one_by_one(gpu_lib, case, own):
     if case == "empty_twice":
         sizes[5] = 0
     orders = [rng.integers(0, n_sku, k).tolist() for k in sizes]
-    plans = cut(rng, len(orders), 160, 9, empty=(4,))      # (enough plans for a shared slotting to come here)
+    plans = cut(rng, len(orders), 24, 9, empty=(4,))
     for k, plan in enumerate(plans):
         if case == "long_unused":
             plan[:] = [[o for o in t if o not in range(40, 45)] for t in plan]
         elif case in ("empty_twice", "twice_in_one"):
-            a, b = (3, 3) if case == "twice_in_one" else (k % 50, 60)
+            a, b = (3, 3) if case == "twice_in_one" else (2 * k, 60)
             plan[a], plan[b] = plan[a] + [5], plan[b] + [5]
         elif case == "all_twice":
-            plan[:] = plan + cut(rng, len(orders), 1, 7)[0]
+            plan[:] = plan + cut(rng, len(orders), 1, 9)[0]
         elif case == "rows_full":                          # the same orders over and over: more lines than the book has
             plan[:] = plan + [t[::-1] for t in plan[:120]] * 2
     inst = make_instance(lay, orders, rng.permutation(lay.n_loc)[:n_sku], plans, n_sku)

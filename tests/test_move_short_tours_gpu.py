@@ -37,23 +37,25 @@ def moves(rng, inst, n):
     return mv
 
 
-@pytest.mark.parametrize("copies", [1, 500])
+COPIES = (1, 500)   # of the moves: four tours a warp and 32
+
+
 @pytest.mark.parametrize("per", [1, 2, 3, 20, 21, 22])
 @pytest.mark.parametrize("lay", [wh_gen.Layout(23, 31), wh_gen.Layout(280, 9, 4, 2, 6)], ids=["narrow", "wide"])
-def test_short_tours(gpu_lib, lay, per, copies):
+def test_short_tours(gpu_lib, lay, per):
     rng = np.random.default_rng(per)
     inst = instance(rng, lay, per)
     maps = np.stack([rng.permutation(lay.n_loc)[:N_SKU] for _ in range(3)]).astype(np.int32)
     mv = moves(rng, inst, 240)
     want_d, want_s = oracle.eval_moves(inst, mv, 0, 0, slot_map=maps.ravel(), slot_map_stride=N_SKU)
     assert (want_s == 0).sum() > 150
-    d, s, st = gpu_moves(gpu_lib, inst, np.tile(mv, (copies, 1)), maps=maps)
-    assert st == 0
-    assert np.array_equal(s, np.tile(want_s, copies)) and np.array_equal(d, np.tile(want_d, (copies, 1)))
+    for copies in COPIES:
+        d, s, st = gpu_moves(gpu_lib, inst, np.tile(mv, (copies, 1)), maps=maps)
+        assert st == 0
+        assert np.array_equal(s, np.tile(want_s, copies)) and np.array_equal(d, np.tile(want_d, (copies, 1)))
 
 
-@pytest.mark.parametrize("copies", [1, 500])
-def test_unusable_lines(gpu_lib, copies):
+def test_unusable_lines(gpu_lib):
     """A line without a usable location gives status 3 to the moves that rewrite its tour, and to no others."""
     rng, lay = np.random.default_rng(9), wh_gen.Layout(23, 31)
     inst = instance(rng, lay, 2)
@@ -72,5 +74,6 @@ def test_unusable_lines(gpu_lib, copies):
         if any(tour_of[1, o] in changed for o in bad):
             want_s[m], want_d[m] = 3, 0
     assert (want_s == 3).sum() > 0
-    d, s, _ = gpu_moves(gpu_lib, inst, np.tile(mv, (copies, 1)), maps=maps, occupancy=False)
-    assert np.array_equal(s, np.tile(want_s, copies)) and np.array_equal(d, np.tile(want_d, (copies, 1)))
+    for copies in COPIES:
+        d, s, _ = gpu_moves(gpu_lib, inst, np.tile(mv, (copies, 1)), maps=maps, occupancy=False)
+        assert np.array_equal(s, np.tile(want_s, copies)) and np.array_equal(d, np.tile(want_d, (copies, 1)))
